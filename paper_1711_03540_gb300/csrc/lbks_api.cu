@@ -1256,6 +1256,7 @@ int lb_ks_load(lb_ks_t* h, const void* buf, size_t bytes) try {
   h->mass0_h = m0;
   h->tables_on_host = true;
   LBKS_CUDA(h, cudaMemcpy(h->d_runs, runs.data(), sizeof(RunDesc) * h->nruns, cudaMemcpyHostToDevice), "load runs");
+  if (h->prec == kF64) LBKS_CUDA(h, launch_fix_coef(h->Q, h->nruns, h->d_runs, h->stream), "load runs");
   LBKS_CUDA(h, cudaMemcpy(h->d_mass0, m0.data(), sizeof(double) * h->nruns, cudaMemcpyHostToDevice), "load mass0");
   LBKS_CUDA(h, cudaMemcpy(h->fbuf[h->cur], p, storage_bytes(h->prec) * (size_t)h->nplanes * (size_t)h->plane,
                           cudaMemcpyHostToDevice), "load populations");

@@ -24,13 +24,20 @@ template <typename CT, int Q> struct Coef {
   CT r, rhobar, scale, inv_scale;
 };
 
+// FP64: the fixed-point coefficients; r, a_i and b_i are read from the run table by the
+// sites that take FP64 arithmetic.
+template <int Q> struct Coef<double, Q> {
+  FixCoef fix;
+  const RunDesc* d;
+  static constexpr double scale = 1.0, inv_scale = 1.0;
+};
+
 template <typename CT, int Q>
 __device__ __forceinline__ Coef<CT, Q> load_coef(const RunDesc& d) {
   Coef<CT, Q> c;
   if constexpr (sizeof(CT) == 8) {
-#pragma unroll
-    for (int i = 0; i < Q; ++i) { c.a[i] = d.a[i]; c.b[i] = d.b[i]; }
-    c.r = d.r; c.rhobar = d.rhobar; c.scale = d.scale; c.inv_scale = d.inv_scale;
+    c.fix = d.fix;
+    c.d = &d;
   } else {
 #pragma unroll
     for (int i = 0; i < Q; ++i) { c.a[i] = d.af[i]; c.b[i] = d.bf[i]; }
@@ -75,8 +82,8 @@ __device__ __forceinline__ CT post_collision(CT r, CT g, CT rho, CT rho2, CT b, 
   return fma_rn(r, g, fma_rn(rho2, b, t));
 }
 
-template <int Q, typename CT>
-__device__ __forceinline__ void collide(CT (&g)[Q], const Coef<CT, Q>& k) {
+template <int Q, typename CT, typename K>
+__device__ __forceinline__ void collide_rn(CT (&g)[Q], const K& k) {
   CT sg = g[0];
 #pragma unroll
   for (int i = 1; i < Q; ++i) sg = add_rn(sg, g[i]);
@@ -92,6 +99,27 @@ __device__ __forceinline__ void collide(CT (&g)[Q], const Coef<CT, Q>& k) {
     acc = add_rn(acc, -g[2 * p]);
   }
   g[0] = acc;
+}
+
+template <int Q>
+__device__ __forceinline__ void collide(float (&g)[Q], const Coef<float, Q>& k) {
+  collide_rn<Q, float>(g, k);
+}
+
+// FP64: in fixed point on the integer pipes (fix_collide); a site it does not cover (a
+// value that is not finite, far out of scale or much smaller than the others) in FP64
+// arithmetic.  Which of the two a site takes depends on its own values alone.
+template <int Q>
+__device__ __forceinline__ void collide(double (&g)[Q], const Coef<double, Q>& k) {
+  uint64_t in[Q], out[Q];
+#pragma unroll
+  for (int i = 0; i < Q; ++i) in[i] = (uint64_t)__double_as_longlong(g[i]);
+  if (fix_collide<Q>(in, out, k.fix)) {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) g[i] = __longlong_as_double((long long)out[i]);
+  } else {
+    collide_rn<Q, double>(g, *k.d);
+  }
 }
 
 __device__ __forceinline__ int64_t wrap_site(int64_t x, int64_t N) {

@@ -5,6 +5,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "lbks_fix64.cuh"
+
 namespace lbks {
 
 constexpr int kMaxQ = 7;
@@ -26,7 +28,14 @@ struct RunDesc {
   double a[8], b[8];  // A_i / tau, B_i / tau
   double A[8], B[8];  // equilibrium coefficients
   double r, rhobar, scale, inv_scale;  // scale: F16S stored value = g / scale
-  float af[8], bf[8];
+  // FP32 copies of a and b; FP64 storage: r, a and b in fixed point (lbks_fix64.cuh),
+  // recomputed on the device whenever a run table is made or loaded
+  union {
+    struct {
+      float af[8], bf[8];
+    };
+    FixCoef fix;
+  };
   float rf, rhobarf, scalef, inv_scalef;
   // Fixed-value ends (front test of Table 5): nodes j <= 0 and j >= N-1, and c_max ghost
   // nodes beyond each end (stored at j = -c_max..-1 and N..N-1+c_max), are reservoirs
@@ -90,6 +99,8 @@ cudaError_t launch_reservoir_step(int Q, int storage, Arena src, Arena dst, cons
 cudaError_t launch_init_stats(int Q, int storage, int nruns, const double* rho0, const int64_t* rho_off,
                               RunDesc* runs, const Tile* tiles, int ntiles, const int32_t* tile_begin,
                               double* partials, double* mass0, int* bad_run, cudaStream_t s);
+// FP64 storage: the fixed-point coefficients of every run, from r, a and b (a loaded run table).
+cudaError_t launch_fix_coef(int Q, int nruns, RunDesc* runs, cudaStream_t s);
 // Guard: per-tile FP64 partial sums of rho and rho^2 (scratch: 2 doubles per tile),
 // then per-run totals, non-finite flag, and (if recentre) g_0 += (M0 - M)/N.
 cudaError_t launch_mass_partials(int Q, int storage, Arena src, const RunDesc* runs, const Tile* tiles,

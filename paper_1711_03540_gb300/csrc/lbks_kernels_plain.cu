@@ -163,16 +163,25 @@ __global__ void __launch_bounds__(kPlainThreads) plain_step_kernel(Arena src, Ar
   if ((int)threadIdx.x >= tl.len) return;
   const RunDesc& d = runs[tl.run];
   const Coef<CT, Q> k = load_coef<CT, Q>(d);
-  const int64_t x = tl.x0 + threadIdx.x;
-  const T* fs = static_cast<const T*>(src.f) + d.off;
-  T* fd = static_cast<T*>(dst.f) + d.off;
+  const int x = tl.x0 + (int)threadIdx.x, N = (int)d.N;
+  const int64_t at = d.off + x;
   CT g[Q];
+  const T* fs = static_cast<const T*>(src.f) + at;
 #pragma unroll
-  for (int i = 0; i < Q; ++i) g[i] = to_compute(fs[(int64_t)i * src.plane + x], k.scale);
-  collide<Q, CT>(g, k);
+  for (int i = 0; i < Q; ++i, fs += src.plane) g[i] = to_compute(*fs, k.scale);
+  collide<Q>(g, k);
+  T* fd = static_cast<T*>(dst.f) + at;
+  constexpr int C = cmax_of(Q);
+  if (tl.x0 >= C && tl.x0 + tl.len + C <= N) {  // no site of the tile streams across the ends
 #pragma unroll
-  for (int i = 0; i < Q; ++i)
-    from_compute(g[i], k.inv_scale, fd + (int64_t)i * dst.plane + wrap_site(x + speed(i), d.N));
+    for (int i = 0; i < Q; ++i, fd += dst.plane) from_compute(g[i], k.inv_scale, fd + speed(i));
+  } else {
+#pragma unroll
+    for (int i = 0; i < Q; ++i, fd += dst.plane) {
+      const int y = x + speed(i);
+      from_compute(g[i], k.inv_scale, fd + (y < 0 ? speed(i) + N : (y >= N ? speed(i) - N : speed(i))));
+    }
+  }
 }
 
 // Lattices with reservoir ends (the fixed end values of the front test, Table 5).
@@ -209,7 +218,7 @@ __global__ void __launch_bounds__(kPlainThreads) reservoir_step_kernel(Arena src
   CT g[Q];
 #pragma unroll
   for (int q = 0; q < Q; ++q) g[q] = to_compute(fs[(int64_t)q * src.plane + j], k.scale);
-  collide<Q, CT>(g, k);
+  collide<Q>(g, k);
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     const int64_t y = j + speed(i);
@@ -483,7 +492,7 @@ __global__ void __launch_bounds__(kPlainThreads) init_stats_partials_kernel(cons
 // M0 (the guard's re-centring target), the mean rhobar = M0 / N that the deviation
 // form stores g_0 against (0 for FP64 storage), and the first run with a non-finite
 // value (atomicMin into bad_run).
-__global__ void init_stats_finalize_kernel(int nruns, int storage, const int32_t* __restrict__ tile_begin,
+__global__ void init_stats_finalize_kernel(int Q, int nruns, int storage, const int32_t* __restrict__ tile_begin,
                                            const double* __restrict__ partials, RunDesc* __restrict__ runs,
                                            double* __restrict__ mass0, int* __restrict__ bad_run) {
   const int run = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -505,7 +514,13 @@ __global__ void init_stats_finalize_kernel(int nruns, int storage, const int32_t
     const double rhobar = storage == kF64 ? 0.0 : m / static_cast<double>(runs[run].N);
     runs[run].rhobar = rhobar;
     runs[run].rhobarf = (float)rhobar;
+    if (storage == kF64) runs[run].fix = fix_coef(Q, runs[run].r, rhobar, runs[run].a, runs[run].b);
   }
+}
+
+__global__ void fix_coef_kernel(int Q, int nruns, RunDesc* __restrict__ runs) {
+  const int run = blockIdx.x * blockDim.x + threadIdx.x;
+  if (run < nruns) runs[run].fix = fix_coef(Q, runs[run].r, runs[run].rhobar, runs[run].a, runs[run].b);
 }
 
 // Scaled FP16 storage, pass 3: per tile the largest |g_i| of the initial state,
@@ -644,13 +659,19 @@ cudaError_t launch_init_stats(int Q, int storage, int nruns, const double* rho0,
   if (ntiles == 0 || nruns == 0) return cudaSuccess;
   const int fin_blocks = (nruns * 32 + 127) / 128;
   init_stats_partials_kernel<<<ntiles, kPlainThreads, 0, s>>>(rho0, rho_off, tiles, partials);
-  init_stats_finalize_kernel<<<fin_blocks, 128, 0, s>>>(nruns, storage, tile_begin, partials, runs, mass0, bad_run);
+  init_stats_finalize_kernel<<<fin_blocks, 128, 0, s>>>(Q, nruns, storage, tile_begin, partials, runs, mass0, bad_run);
   if (storage == kF16S) {
     if (Q == 5) init_scale_partials_kernel<5><<<ntiles, kPlainThreads, 0, s>>>(rho0, rho_off, runs, tiles, partials);
     else if (Q == 7) init_scale_partials_kernel<7><<<ntiles, kPlainThreads, 0, s>>>(rho0, rho_off, runs, tiles, partials);
     else return cudaErrorInvalidValue;
     init_scale_finalize_kernel<<<fin_blocks, 128, 0, s>>>(nruns, tile_begin, partials, runs);
   }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fix_coef(int Q, int nruns, RunDesc* runs, cudaStream_t s) {
+  if (nruns == 0) return cudaSuccess;
+  fix_coef_kernel<<<(nruns + 127) / 128, 128, 0, s>>>(Q, nruns, runs);
   return cudaGetLastError();
 }
 

@@ -152,7 +152,7 @@ __device__ __forceinline__ void stream_step(Arena src, Arena dst, const RunDesc*
             g[u][i] = (k0 + u < len) ? to_compute(fs[(int64_t)i * src.plane + x0 + k0 + u], k.scale) : CT(0);
       }
 #pragma unroll
-      for (int u = 0; u < kVec; ++u) collide<Q, CT>(g[u], k);
+      for (int u = 0; u < kVec; ++u) collide<Q>(g[u], k);
       if (k0 + kVec <= len) {
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
@@ -175,7 +175,7 @@ __device__ __forceinline__ void stream_step(Arena src, Arena dst, const RunDesc*
       CT g[Q];
 #pragma unroll
       for (int i = 0; i < Q; ++i) g[i] = to_compute(fs[(int64_t)i * src.plane + xs], k.scale);
-      collide<Q, CT>(g, k);
+      collide<Q>(g, k);
 #pragma unroll
       for (int i = 0; i < Q; ++i) put(&sm[i * W + col], g[i], k.inv_scale);
     }

@@ -256,6 +256,22 @@ __device__ __forceinline__ void push_edge_left(const CT (&f)[Q][S], const CT (&r
   });
 }
 
+// The same for FP64, whose post-collision values are already in f: the last k + 1 slots of
+// each plane of speed +k (RIGHT), or the first k + 1 of each of speed -k.
+template <int Q, bool RIGHT, typename CT, int S>
+__device__ __forceinline__ void push_edge(const CT (&f)[Q][S], uint32_t col, int ntx) {
+  StaticFor<1, Q>::run([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    constexpr int c = speed(i);
+    constexpr int kk = c > 0 ? c : -c;
+    if constexpr ((c > 0) == RIGHT) {
+#pragma unroll
+      for (int j = 0; j <= kk; ++j)
+        st_cluster(col + (uint32_t)((xrow(kk) + j) * ntx * sizeof(CT)), f[i][RIGHT ? S - 1 - kk + j : j]);
+    }
+  });
+}
+
 // Link state of a block of a cluster pair whose bundle has a piece across the block
 // edge: the thread's links to the other block, this block's mbarriers (one per step
 // parity), the other block's exchange area and mbarriers in the cluster window, the
@@ -304,66 +320,111 @@ __device__ __forceinline__ void resident_steps(CT (&f)[Q][S], const Coef<CT, Q>&
     CT* const xp = xbase + pb * 2 * NR * NTX;  // this step's exchange area: [R|L][NR][NTX]
     CT* const xw = xp + t;                     // this thread's column
     if (!SKIP || active) {
-      // A. per-site sums; g_0's register becomes the accumulator of g*_0
-      CT rho[S], rho2[S], tt[S];
+      if constexpr (sizeof(CT) == 8) {
+        // FP64: each site collides as a whole (its planes share one fixed-point grid), in
+        // place; then the edge values go out and the planes move along in the registers.
 #pragma unroll
-      for (int s = 0; s < S; ++s) {
-        CT sg = f[0][s];
+        for (int s = 0; s < S; ++s) {
+          CT g[Q];
 #pragma unroll
-        for (int i = 1; i < Q; ++i) sg = add_rn(sg, f[i][s]);
-        rho[s] = add_rn(k.rhobar, sg);
-        rho2[s] = mul_rn(rho[s], rho[s]);
-        f[0][s] = sg;
-      }
-      if constexpr (LINK) {
-        // Send the values this step sends across the block edge before phase B, from
-        // phase A's sums with the arithmetic of phase B (which computes them again
-        // below), so that the transfer overlaps the rest of the step; each sending
-        // thread then arrives on the other block's mbarrier of this parity, releasing its
-        // stores at cluster scope (this step's phase there completes on the two
-        // arrivals, one per direction).  Arriving after phase B instead delays the
-        // receiver: 7 % slower rings.
-        if (step != ln.withhold) {
-          if (ln.rrem) {
-            push_edge_right<Q>(f, rho, rho2, k, ln.peer_x + (uint32_t)((pb * 2 * NR * NTX + XS - 2) * sizeof(CT)),
-                               NTX);
-            mbar_arrive_remote(ln.peer_mbar + 8u * pb);
-          }
-          if (ln.lrem) {
-            push_edge_left<Q>(f, rho, rho2, k,
-                              ln.peer_x + (uint32_t)(((pb * 2 + 1) * NR * NTX + XS - 1) * sizeof(CT)), NTX);
-            mbar_arrive_remote(ln.peer_mbar + 8u * pb);
+          for (int i = 0; i < Q; ++i) g[i] = f[i][s];
+          collide<Q>(g, k);
+#pragma unroll
+          for (int i = 0; i < Q; ++i) f[i][s] = g[i];
+        }
+        if constexpr (LINK) {
+          if (step != ln.withhold) {
+            if (ln.rrem) {
+              push_edge<Q, true>(f, ln.peer_x + (uint32_t)((pb * 2 * NR * NTX + XS - 2) * sizeof(CT)), NTX);
+              mbar_arrive_remote(ln.peer_mbar + 8u * pb);
+            }
+            if (ln.lrem) {
+              push_edge<Q, false>(f, ln.peer_x + (uint32_t)(((pb * 2 + 1) * NR * NTX + XS - 1) * sizeof(CT)), NTX);
+              mbar_arrive_remote(ln.peer_mbar + 8u * pb);
+            }
           }
         }
-      }
-      // B. plane by plane: collide, write to the destination site's register and/or the
-      // exchange column.
-      StaticFor<1, Q>::run([&](auto ic) {
-        constexpr int i = decltype(ic)::value;
-        constexpr int c = speed(i);
-        constexpr int kk = c > 0 ? c : -c;
-        constexpr int row0 = xrow(kk);
-        if constexpr (c > 0) {
+        StaticFor<1, Q>::run([&](auto ic) {
+          constexpr int i = decltype(ic)::value;
+          constexpr int c = speed(i);
+          constexpr int kk = c > 0 ? c : -c;
+          constexpr int row0 = xrow(kk);
+          if constexpr (c > 0) {
 #pragma unroll
-          for (int s = S - 1; s >= 0; --s) {
-            tt[s] = mul_rn(rho[s], k.a[i]);  // shared with the -c plane that follows
-            const CT v = post_collision(k.r, f[i][s], rho[s], rho2[s], k.b[i], tt[s]);
-            f[0][s] = add_rn(f[0][s], -v);
-            if (s >= S - 1 - kk) xw[(row0 + s - (S - 1 - kk)) * NTX] = v;
-            if (s + kk <= S - 1) f[i][s + kk] = v;
+            for (int s = S - 1; s >= 0; --s) {
+              if (s >= S - 1 - kk) xw[(row0 + s - (S - 1 - kk)) * NTX] = f[i][s];
+              if (s + kk <= S - 1) f[i][s + kk] = f[i][s];
+            }
+          } else {
+#pragma unroll
+            for (int s = 0; s < S; ++s) {
+              if (s <= kk) xw[(NR + row0 + s) * NTX] = f[i][s];
+              if (s >= kk) f[i][s - kk] = f[i][s];
+            }
           }
-        } else {
+        });
+      } else {
+        // A. per-site sums; g_0's register becomes the accumulator of g*_0
+        CT rho[S], rho2[S], tt[S];
 #pragma unroll
-          for (int s = 0; s < S; ++s) {
-            // b_i of the -c plane is exactly minus the +c plane's (B_i = J w1_i, w1 odd in
-            // c), taken with the FMA's negation so that it needs no register of its own
-            const CT v = post_collision(k.r, f[i][s], rho[s], rho2[s], -k.b[i - 1], tt[s]);
-            f[0][s] = add_rn(f[0][s], -v);
-            if (s <= kk) xw[(NR + row0 + s) * NTX] = v;
-            if (s >= kk) f[i][s - kk] = v;
+        for (int s = 0; s < S; ++s) {
+          CT sg = f[0][s];
+#pragma unroll
+          for (int i = 1; i < Q; ++i) sg = add_rn(sg, f[i][s]);
+          rho[s] = add_rn(k.rhobar, sg);
+          rho2[s] = mul_rn(rho[s], rho[s]);
+          f[0][s] = sg;
+        }
+        if constexpr (LINK) {
+          // Send the values this step sends across the block edge before phase B, from
+          // phase A's sums with the arithmetic of phase B (which computes them again
+          // below), so that the transfer overlaps the rest of the step; each sending
+          // thread then arrives on the other block's mbarrier of this parity, releasing its
+          // stores at cluster scope (this step's phase there completes on the two
+          // arrivals, one per direction).  Arriving after phase B instead delays the
+          // receiver: 7 % slower rings.
+          if (step != ln.withhold) {
+            if (ln.rrem) {
+              push_edge_right<Q>(f, rho, rho2, k, ln.peer_x + (uint32_t)((pb * 2 * NR * NTX + XS - 2) * sizeof(CT)),
+                                 NTX);
+              mbar_arrive_remote(ln.peer_mbar + 8u * pb);
+            }
+            if (ln.lrem) {
+              push_edge_left<Q>(f, rho, rho2, k,
+                                ln.peer_x + (uint32_t)(((pb * 2 + 1) * NR * NTX + XS - 1) * sizeof(CT)), NTX);
+              mbar_arrive_remote(ln.peer_mbar + 8u * pb);
+            }
           }
         }
-      });
+        // B. plane by plane: collide, write to the destination site's register and/or the
+        // exchange column.
+        StaticFor<1, Q>::run([&](auto ic) {
+          constexpr int i = decltype(ic)::value;
+          constexpr int c = speed(i);
+          constexpr int kk = c > 0 ? c : -c;
+          constexpr int row0 = xrow(kk);
+          if constexpr (c > 0) {
+#pragma unroll
+            for (int s = S - 1; s >= 0; --s) {
+              tt[s] = mul_rn(rho[s], k.a[i]);  // shared with the -c plane that follows
+              const CT v = post_collision(k.r, f[i][s], rho[s], rho2[s], k.b[i], tt[s]);
+              f[0][s] = add_rn(f[0][s], -v);
+              if (s >= S - 1 - kk) xw[(row0 + s - (S - 1 - kk)) * NTX] = v;
+              if (s + kk <= S - 1) f[i][s + kk] = v;
+            }
+          } else {
+#pragma unroll
+            for (int s = 0; s < S; ++s) {
+              // b_i of the -c plane is exactly minus the +c plane's (B_i = J w1_i, w1 odd in
+              // c), taken with the FMA's negation so that it needs no register of its own
+              const CT v = post_collision(k.r, f[i][s], rho[s], rho2[s], -k.b[i - 1], tt[s]);
+              f[0][s] = add_rn(f[0][s], -v);
+              if (s <= kk) xw[(NR + row0 + s) * NTX] = v;
+              if (s >= kk) f[i][s - kk] = v;
+            }
+          }
+        });
+      }
     }
     if constexpr (kLeave) named_barrier(1, nbar);
     else __syncthreads();
