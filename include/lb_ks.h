@@ -79,7 +79,7 @@ extern "C" {
 
 /* Kernel family. */
 #define LB_KS_KERNEL_AUTO 0     /* resident when every run fits its constraints, else plain (F64) / stream */
-#define LB_KS_KERNEL_PLAIN 1    /* one thread per site, one launch per step (F64, F32) */
+#define LB_KS_KERNEL_PLAIN 1    /* one thread per site, one launch per step (F64, F32); reservoir ends: many steps per launch */
 #define LB_KS_KERNEL_STREAM 2   /* HBM-streaming tiles, one launch per step (F32, F16S) */
 #define LB_KS_KERNEL_RESIDENT 3 /* register-resident, many steps per launch (F64, F32, F16S) */
 /* tau = 1 only (every run): at tau = 1 the BGK collision of Eq. LB_equation_ordinary
@@ -273,7 +273,8 @@ LB_KS_API int64_t lb_ks_steps_done(const lb_ks_t *h);
 
 /*
  * Describe the handle: kernel family actually used (LB_KS_KERNEL_*), resident
- * sites per thread, threads per block, steps per launch and blocks per work group
+ * sites per thread (1: the one-site-per-thread resident kernel, the automatic choice for
+ * F64 and for F32 batches too small to fill the device), threads per block, steps per launch and blocks per work group
  * of whole lattices (1 or 2; all 0 when not resident), number of runs and total
  * sites.  Any pointer may be NULL.
  */

@@ -63,6 +63,7 @@ struct Lane {
   int kx = 0;  // cl = 2: steps between the halo exchanges of lattice halves
   bool merged = false;  // cl = 2: single-block bundles run two to a pair work group
   int halves = 0;       // lattices held as two halves
+  bool one = false;     // every bundle holds one piece
   Piece* d_pieces = nullptr;
   int2* d_bundles = nullptr;
   int* d_queue = nullptr;
@@ -95,6 +96,7 @@ using RunTable = std::vector<RunDesc, NoInitAlloc<RunDesc>>;
 struct lb_ks {
   int Q = 0, prec = 0, kernel = 0, cmax = 0;
   int nplanes = 0;         // stored planes: Q, or 1 for the tau = 1 collapse (rho - rhobar)
+  bool blocked = false;  // one site per thread, many steps per launch (one lane, S = 1)
   bool collapse_resident = false;  // tau = 1 collapse on its register-resident kernel (lanes below)
   bool reservoir = false;  // lattices with fixed-value ends instead of periodic ones
   lb_ks_opts opts{};
@@ -286,11 +288,8 @@ int default_threads(int prec, int S) {
   return S <= 8 ? 512 : (S <= 12 ? 384 : 256);
 }
 
-int upload_lane(lb_ks* h, Lane* L, const std::vector<Piece>& pieces, const Bins& bins, int cl, int k, bool segmented,
-                double weight) {
-  std::vector<Piece> ordered;
-  std::vector<int2> bundles;
-  bins.emit(pieces, &ordered, &bundles);
+int upload_lane(lb_ks* h, Lane* L, const std::vector<Piece>& ordered, const std::vector<int2>& bundles, int cl, int k,
+                bool segmented, double weight) {
   L->cl = cl;
   L->segmented = segmented;
   L->weight = weight;
@@ -305,9 +304,17 @@ int upload_lane(lb_ks* h, Lane* L, const std::vector<Piece>& pieces, const Bins&
   return LB_KS_OK;
 }
 
+int upload_lane(lb_ks* h, Lane* L, const std::vector<Piece>& pieces, const Bins& bins, int cl, int k, bool segmented,
+                double weight) {
+  std::vector<Piece> ordered;
+  std::vector<int2> bundles;
+  bins.emit(pieces, &ordered, &bundles);
+  return upload_lane(h, L, ordered, bundles, cl, k, segmented, weight);
+}
+
 // The kernels' launch preparation (dynamic shared memory opt-in, resident blocks per SM
 // or clusters at once), done once per device, kind (0 resident, 1 collapse, 2 cluster
-// pairs), scheme, storage and tiling: the attribute set by it stays with the function.
+// pairs, 3 and 4 one site per thread, periodic and reservoir), scheme, storage and tiling: the attribute set by it stays with the function.
 cudaError_t prepared(int kind, int Q, int prec, int S, int NT, int* out) {
   static std::mutex mu;
   static std::map<std::array<int, 6>, int> done;
@@ -320,12 +327,62 @@ cudaError_t prepared(int kind, int Q, int prec, int S, int NT, int* out) {
   if (it == done.end()) {
     int v = 0;
     e = kind == 0 ? resident_prepare(Q, prec, S, NT, &v)
-                  : (kind == 1 ? collapse_resident_prepare(Q, prec, S, NT, &v) : resident_cluster_prepare(Q, prec, S, NT, &v));
+        : kind == 1 ? collapse_resident_prepare(Q, prec, S, NT, &v)
+        : kind == 2 ? resident_cluster_prepare(Q, prec, S, NT, &v)
+                    : blocked_prepare(Q, prec, NT, kind == 4, &v);
     if (e != cudaSuccess) return e;  // not kept: the caller clears the error and tries another tiling
     it = done.emplace(key, v).first;
   }
   *out = it->second;
   return cudaSuccess;
+}
+
+// Plan of the blocked kernel (one site per thread): LB_KS_OK, 1 if the plan is not the
+// blocked kernel's (`always` = false and the register-resident kernel is estimated
+// faster), or an error.
+int setup_blocked(lb_ks* h, bool always) {
+  int dev = 0, sms = 0;
+  LBKS_CUDA(h, cudaGetDevice(&dev), "cudaGetDevice");
+  LBKS_CUDA(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute");
+  const int R = h->opts.recentre_every;
+  const BlockedTiling b =
+      choose_blocked(h->N, h->reservoir, h->Q, h->prec == kF64, sms, R > 0 ? std::min(R, 1000) : 1000);
+  if (b.NT == 0) return 1;
+  // FP32: a step of the register-resident kernel takes 0.88 us with its 5120-site blocks at
+  // most one per SM (0.47 us with one warp per scheduler), more in proportion beyond that
+  if (!always && h->prec != kF64) {
+    const double fill = (double)h->total_sites / (5120.0 * sms);
+    if (b.us > (h->Q == 7 ? 0.88 : 0.62) * std::max(1.0, 1.1 * fill)) return 1;
+  }
+  std::vector<Piece> pieces;
+  if (!plan_blocked(h->N, h->reservoir, h->cmax, b.NT, b.k, &pieces)) return 1;
+  int bps = 0;
+  cudaError_t e = prepared(h->reservoir ? 4 : 3, h->Q, h->prec, 1, b.NT, &bps);
+  if (e != cudaSuccess || bps < 1) { cudaGetLastError(); return 1; }
+  std::vector<Piece> ordered;
+  std::vector<int2> bundles;
+  blocked_bundles(pieces, b.NT, b.spread, &ordered, &bundles);
+  bool segmented = false;
+  for (const Piece& p : pieces) segmented = segmented || p.st_hi - p.st_lo < p.n;
+  Lane& L = h->lanes[0];
+  int rc;
+  if ((rc = upload_lane(h, &L, ordered, bundles, 1, b.k, segmented, 1.0))) return rc;
+  L.grid = L.nbundles;
+  L.one = bundles.size() == pieces.size();
+  h->nlanes = 1;
+  h->blocked = true;
+  h->S = 1;
+  h->NT = b.NT;
+  h->kmax = h->kseg = b.k;
+  return LB_KS_OK;
+}
+
+// Whether the blocked kernel may run a periodic handle: no tiling asked for, and a storage
+// that is not rounded at launch edges (scaled FP16 is).
+bool blocked_eligible(const lb_ks* h) {
+  const lb_ks_opts& o = h->opts;
+  return h->nplanes != 1 && h->prec != kF16S && !o.sites_per_thread && !o.threads_per_block && !o.steps_per_launch &&
+         !o.cluster_size;
 }
 
 // Resident kernel plan.  Whole lattices (rings) run k_ring steps per launch; lattices
@@ -344,6 +401,11 @@ cudaError_t prepared(int kind, int Q, int prec, int S, int NT, int* out) {
 int setup_resident(lb_ks* h, bool required, int S_force = 0, int NT_force = 0, double lane_weight = 1.25,
                    int cl_force = 0, int merge = -1, int kx_force = -1) {
   const bool col = h->nplanes == 1;  // the tau = 1 collapse's resident kernel
+  h->blocked = false;
+  if (S_force == 1 || (S_force == 0 && blocked_eligible(h))) {
+    const int rc = setup_blocked(h, S_force == 1);
+    if (rc <= 0 || S_force == 1) return rc;
+  }
   auto supported = [&](int S, int NT) {
     return col ? collapse_resident_supported(h->Q, h->prec, S, NT) : resident_supported(h->Q, h->prec, S, NT);
   };
@@ -451,11 +513,11 @@ int issue_lane(lb_ks* h, const Lane& L, int64_t k, int from, bool in_place, cuda
   while (k > 0) {
     const int64_t kk = std::min<int64_t>(k, L.k);
     const int dst = (in_place && kk == k && cur == from) ? cur : 1 - cur;
-    LBKS_CUDA(h, cudaMemsetAsync(L.d_queue, 0, sizeof(int), s), "queue reset");
+    if (!h->blocked) LBKS_CUDA(h, cudaMemsetAsync(L.d_queue, 0, sizeof(int), s), "queue reset");
     ResidentLaunch RL{h->Q, h->prec, h->S, h->NT, arena(h, cur), arena(h, dst), h->d_runs,
                       L.d_pieces, L.d_bundles, L.nbundles, L.d_queue, (int)kk, L.grid, L.cl, h->d_flags,
-                      h->nplanes == 1, L.kx, h->link_wait_limit, h->link_withhold_step};
-    LBKS_CUDA(h, launch_resident(RL, s), "resident step");
+                      h->nplanes == 1, L.kx, h->link_wait_limit, h->link_withhold_step, L.one};
+    LBKS_CUDA(h, h->blocked ? launch_blocked(RL, h->reservoir, s) : launch_resident(RL, s), "resident step");
     *nk += 1;
     cur = dst;
     k -= kk;
@@ -485,7 +547,7 @@ int issue_steps(lb_ks* h, int64_t n, cudaStream_t s, int64_t* nk) {
   const int64_t R = h->opts.recentre_every;
   while (n > 0) {
     int64_t k = 1;
-    if (h->kernel == LB_KS_KERNEL_RESIDENT || h->collapse_resident) {
+    if (h->nlanes > 0) {
       k = std::min<int64_t>(n, h->kmax);
       if (R > 0) k = std::min<int64_t>(k, R - h->phase);
       int to = h->cur, rc;
@@ -614,6 +676,7 @@ int autotune_resident(lb_ks* h) {
   std::vector<Cand> cands;
   std::vector<std::pair<int, int>> tilings;
   const bool col = h->nplanes == 1;  // the tau = 1 collapse's resident kernel
+  if (blocked_eligible(h)) cands.push_back({1, 0, 1.0, 1, 0, 0});  // one site per thread
   if (h->opts.sites_per_thread) {
     tilings.push_back({h->opts.sites_per_thread, h->opts.threads_per_block});
   } else if (col) {
@@ -959,6 +1022,7 @@ int create_body(lb_ks*& h, lb_ks_t** out, int scheme, int32_t nruns, const int64
     }
   } else if (reservoir) {
     kern = LB_KS_KERNEL_PLAIN;
+    if (h->prec != kF16S && (rc = setup_blocked(h, true)) < 0) return bail(rc);
   } else if (kern == LB_KS_KERNEL_AUTO || kern == LB_KS_KERNEL_RESIDENT) {
     rc = setup_resident(h, kern == LB_KS_KERNEL_RESIDENT);
     if (rc < 0) return bail(rc);
@@ -1074,7 +1138,7 @@ int lb_ks_step(lb_ks_t* h, int64_t n) try {
   if (h->sticky) return h->sticky;
   if (n < 0) return fail(h, LB_KS_EINVAL, "n must be >= 0");
   const int64_t R = h->opts.recentre_every;
-  const int64_t chunk_max = (h->kernel == LB_KS_KERNEL_RESIDENT || h->collapse_resident) ? 64LL * h->kmax : 512;
+  const int64_t chunk_max = h->nlanes > 0 ? 64LL * h->kmax : 512;
   while (n > 0) {
     int64_t c = std::min(n, chunk_max);
     if (R > 0) c = std::min<int64_t>(c, R - h->phase);

@@ -127,6 +127,7 @@ struct ResidentLaunch {
   int kx = 0;             // cl = 2: steps between the halo exchanges of lattice halves (Piece::halo)
   uint32_t wait_limit = 1u << 22;  // cl = 2: try_wait rounds before a wait on the other block gives up
   int withhold_step = -1;          // cl = 2, testing aid: block 1 sends nothing across the edge at this step
+  bool one = false;                // blocked kernel: every bundle holds one piece
 };
 bool resident_supported(int Q, int storage, int S, int NT);
 cudaError_t resident_prepare(int Q, int storage, int S, int NT, int* blocks_per_sm);
@@ -144,6 +145,12 @@ cudaError_t launch_collapse_resident(const ResidentLaunch& L, cudaStream_t s);
 cudaError_t resident_cluster_prepare(int Q, int storage, int S, int NT, int* max_clusters);
 cudaError_t launch_resident_cluster(const ResidentLaunch& L, cudaStream_t s);
 cudaError_t launch_resident(const ResidentLaunch& L, cudaStream_t s);
+
+// One site per thread, ksteps steps per launch (lbks_kernels_blocked.cu): bundles of
+// pieces, one block each (ResidentLaunch::nbundles blocks, no queue).
+bool blocked_supported(int Q, int storage, int NT);
+cudaError_t blocked_prepare(int Q, int storage, int NT, bool reservoir, int* blocks_per_sm);
+cudaError_t launch_blocked(const ResidentLaunch& L, bool reservoir, cudaStream_t s);
 
 // Diagnostic micro-benchmark of the FMA pipes (flop/s), used by the benchmark
 // to state measured ALU peaks beside the derived ones.

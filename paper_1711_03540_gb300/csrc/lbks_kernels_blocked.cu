@@ -1,0 +1,174 @@
+// Temporally blocked step with one site per thread: many steps per launch.
+//
+// A block holds one or more pieces (Piece, thread t0 + j holds the piece's site j): whole
+// lattices (rings), or stretches of longer ones with c_max ksteps halo sites on each side.
+// Every thread keeps its site's Q populations in registers.  One step: collide, write the
+// Q - 1 moving planes to the exchange area in shared memory (double-buffered by step
+// parity), one block barrier, read plane i from the thread holding site x - c_i of the
+// piece (its ends wrap: the periodic ring, or for a stretch values that travel c_max sites
+// per step and stop short of the stored middle).
+//
+// Lattices with reservoir ends: the piece's nodes may include the fixed ones (j <= 0,
+// j >= N - 1 and c_max ghosts beyond each end).  They collide the values they hold and
+// then hold f^eq of the end's density, so from the third step on their exchange values,
+// in both parities, do not change.
+//
+// When and why.  FP64 storage by default (also with reservoir ends): the fixed-point
+// collision needs many warps to hide its latencies, which the register-resident kernel's
+// several sites per thread leave no registers for (8 warps an SM against 24 here), and a
+// single lattice is spread over the SMs instead of sitting on one or two.  FP32 storage
+// when the batch is too small to give every SM a full register-resident block
+// (choose_blocked in lbks_plan.h, setup_blocked): one 4096-site lattice takes 0.18 us per
+// step in stretches over 64 SMs against 0.88 us in one block, 2^18 sites 0.88 against
+// 1.12 us; 2^20 sites 3.1 against 2.2 us, so large FP32 batches stay register-resident.
+// Not for scaled FP16, whose results depend on where launches end (rounded there).
+// Per step and stretch: the halos cost 2 c_max k of NT sites, a launch 1.5 to 2 us in all.
+// Measured (GB300): one 4096-site D1Q7 FP64 lattice 16.8 -> 0.75 us per step (stretches of
+// 32 sites, 16 steps per launch; bound by the latency of one warp's collision), the
+// 4096-lattice FP64 ensemble 615 -> 219 us per step, 4.3e10 site-updates/s (256 threads, 4
+// steps per launch; bound by the integer pipe, 54 % busy, and the conversions, 56 %), 122
+// front lattices 9.3 -> 2.3 us per step, 24 FP32 lattices 0.87 -> 0.37 us per step.
+#include "lbks_device.cuh"
+#include "lbks_plan.h"
+
+namespace lbks {
+
+namespace {
+
+using plan::kBlockedPieces;
+
+template <int Q, int ST> struct BlockedCfg {
+  static constexpr int kMaxThreads = ST == kF64 ? 384 : 512;
+  // blocks of kMaxThreads an SM holds: sets the register budget (80 and 64)
+  static constexpr int kMinBlocks = 2;
+  // Row of the exchange area, a compile-time stride: a column per thread.  FP64: and, for
+  // each piece, c_max on either side of its own, where the threads at the piece's other end
+  // put the values that wrap, so that every access is one address plus an immediate and no
+  // registers are held for the neighbours.  FP32 has the registers: the six neighbours'
+  // columns are computed once, which takes fewer instructions per step.
+  static constexpr bool kGuard = ST == kF64;
+  static constexpr int kXS = kMaxThreads + (kGuard ? 2 * cmax_of(Q) * kBlockedPieces : 0);
+};
+
+// ONE: every bundle holds one piece.
+template <int Q, int ST, bool RES, bool ONE>
+__global__ void __launch_bounds__(BlockedCfg<Q, ST>::kMaxThreads, BlockedCfg<Q, ST>::kMinBlocks)
+    blocked_step_kernel(Arena src, Arena dst, const RunDesc* __restrict__ runs, const Piece* __restrict__ pieces,
+                        const int2* __restrict__ bundles, int ksteps) {
+  using T = typename StorageType<ST>::type;
+  using CT = typename StorageType<ST>::compute;
+  constexpr int C = cmax_of(Q), XS = BlockedCfg<Q, ST>::kXS;
+  constexpr bool kGuard = BlockedCfg<Q, ST>::kGuard;
+  __shared__ CT ex[2][Q - 1][XS];  // [step parity][plane i - 1]
+  // (the pieces are written once, before any launch)
+  const int t = threadIdx.x;
+  int p = blockIdx.x, q = 0;
+  if constexpr (!ONE) {
+    const int2 bd = bundles[blockIdx.x];
+    p = bd.x;
+    for (int u = 1; u < bd.y; ++u)
+      if (t >= pieces[bd.x + u].t0) q = u;
+    p += q;
+  }
+  const Piece pc = pieces[p];
+  const int n = pc.n, j = t - pc.t0;
+  const bool active = j < n;
+  wait_prior_grid();
+  const RunDesc& d = runs[pc.run];
+  int x = (int)pc.x0 + j;  // run-local site (N <= 2^30)
+  bool fixed = false;
+  if constexpr (RES) fixed = x <= 0 || x >= (int)d.N - 1;
+  else if (x >= (int)d.N) x -= (int)d.N;
+  CT g[Q];
+  if (active) {
+    const T* fs = static_cast<const T*>(src.f) + d.off + x;
+#pragma unroll
+    for (int i = 0; i < Q; ++i, fs += src.plane) g[i] = *fs;
+  }
+  const Coef<CT, Q> k = load_coef<CT, Q>(d);
+  CT* const own = &ex[0][0][t + (kGuard ? C * (2 * q + 1) : 0)];
+  int from[Q];  // plane i's new value: the column of the thread holding x - c_i, less this one's
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    const int c = (i + 1) / 2;
+    from[i] = (i & 1) ? (j >= c ? -c : n - c) : (j + c < n ? c : c - n);
+  }
+  for (int s = 0; s < ksteps; ++s) {
+    CT* const xs = own + (s & 1) * (Q - 1) * XS;
+    if (active && (!RES || !fixed || s < 3)) {
+      collide<Q>(g, k);
+#pragma unroll
+      for (int i = 1; i < Q; ++i) {
+        const int c = (i + 1) / 2;
+        CT* const w = xs + (i - 1) * XS;
+        *w = g[i];
+        // the last c sites' right-moving values enter at the piece's start, and so on
+        if (kGuard && ((i & 1) ? j >= n - c : j < c)) w[(i & 1) ? -n : n] = g[i];
+      }
+      if constexpr (RES) {
+        if (fixed) {
+          const double rb = x <= 0 ? d.rho_left : d.rho_right;
+#pragma unroll
+          for (int i = 0; i < Q; ++i) {
+            double v = __fma_rn(d.B[i], __dmul_rn(rb, rb), __dmul_rn(d.A[i], rb));
+            if (i == 0) v = __dsub_rn(v, d.rhobar);
+            g[i] = static_cast<CT>(v);
+          }
+        }
+      }
+    }
+    __syncthreads();
+    if (active && !fixed) {
+#pragma unroll
+      for (int i = 1; i < Q; ++i) g[i] = xs[(i - 1) * XS + (kGuard ? -speed(i) : from[i])];
+    }
+  }
+  if (active && j >= pc.st_lo && j < pc.st_hi) {
+    T* fd = static_cast<T*>(dst.f) + d.off + x;
+#pragma unroll
+    for (int i = 0; i < Q; ++i, fd += dst.plane) *fd = g[i];
+  }
+}
+
+template <int Q, int ST, bool RES>
+cudaError_t prepare_t(int NT, int* blocks_per_sm) {
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, blocked_step_kernel<Q, ST, RES, false>, NT, 0);
+}
+
+template <int Q, int ST, bool RES>
+cudaError_t launch_t(const ResidentLaunch& L, cudaStream_t s) {
+  return launch_early(L.one ? blocked_step_kernel<Q, ST, RES, true> : blocked_step_kernel<Q, ST, RES, false>, L.nbundles,
+                      L.NT, 0, s, L.src, L.dst, L.runs, L.pieces, L.bundles, L.ksteps);
+}
+
+#define LBKS_BLOCKED_DISPATCH(OP)                                                    \
+  do {                                                                               \
+    if (Q == 5 && storage == kF64) { constexpr int Qc = 5, STc = kF64; OP; }         \
+    if (Q == 5 && storage == kF32) { constexpr int Qc = 5, STc = kF32; OP; }         \
+    if (Q == 7 && storage == kF64) { constexpr int Qc = 7, STc = kF64; OP; }         \
+    if (Q == 7 && storage == kF32) { constexpr int Qc = 7, STc = kF32; OP; }         \
+  } while (0)
+
+}  // namespace
+
+bool blocked_supported(int Q, int storage, int NT) {
+  return (Q == 5 || Q == 7) && (storage == kF64 || storage == kF32) && NT >= 32 && NT <= (storage == kF64 ? 384 : 512) && NT % 32 == 0;
+}
+
+cudaError_t blocked_prepare(int Q, int storage, int NT, bool reservoir, int* blocks_per_sm) {
+  if (!blocked_supported(Q, storage, NT)) return cudaErrorInvalidValue;
+  if (reservoir) LBKS_BLOCKED_DISPATCH(return (prepare_t<Qc, STc, true>(NT, blocks_per_sm)));
+  else LBKS_BLOCKED_DISPATCH(return (prepare_t<Qc, STc, false>(NT, blocks_per_sm)));
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_blocked(const ResidentLaunch& L, bool reservoir, cudaStream_t s) {
+  const int Q = L.Q, storage = L.storage;
+  if (!blocked_supported(Q, storage, L.NT)) return cudaErrorInvalidValue;
+  if (L.nbundles == 0) return cudaSuccess;
+  if (reservoir) LBKS_BLOCKED_DISPATCH(return (launch_t<Qc, STc, true>(L, s)));
+  else LBKS_BLOCKED_DISPATCH(return (launch_t<Qc, STc, false>(L, s)));
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace lbks

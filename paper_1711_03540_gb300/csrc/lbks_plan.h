@@ -5,6 +5,7 @@
 #pragma once
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <initializer_list>
 #include <utility>
@@ -125,6 +126,113 @@ inline bool plan_pieces(const std::vector<int64_t>& Ns, int C, int S, int NT, in
     }
   }
   return true;
+}
+
+// Pieces a block of the one-site-per-thread kernel holds at most (plan_blocked gives each
+// at least its share of the block's threads).
+constexpr int kBlockedPieces = 16;
+
+// Pieces of every run for one site per thread: lattices of up to NT sites whole, longer
+// ones in equal stretches with C k halo sites on each side.  Reservoir lattices cover the
+// nodes [-C, N + C), their stretches' halos end there.  False if NT holds no stretch.
+inline bool plan_blocked(const std::vector<int64_t>& Ns, bool reservoir, int C, int NT, int64_t k,
+                         std::vector<Piece>* pieces) {
+  pieces->clear();
+  const int64_t ghost = reservoir ? C : 0;
+  for (int32_t r = 0; r < (int32_t)Ns.size(); ++r) {
+    const int64_t n = Ns[r] + 2 * ghost;
+    if (n <= NT) {
+      Piece p{};
+      p.run = r; p.n = (int)n; p.x0 = -ghost; p.st_hi = (int)n;
+      p.nthr = std::max(p.n, NT / kBlockedPieces);
+      pieces->push_back(p);
+      continue;
+    }
+    const int64_t h = C * k, room = NT - 2 * h;
+    if (room <= 0) return false;
+    const int64_t nseg = (n + room - 1) / room, len = (n + nseg - 1) / nseg;
+    for (int64_t s0 = 0; s0 < n; s0 += len) {
+      const int64_t s1 = std::min(s0 + len, n);
+      const int64_t lo = reservoir ? std::max<int64_t>(s0 - h, 0) : s0 - h;
+      const int64_t hi = reservoir ? std::min(s1 + h, n) : s1 + h;
+      Piece p{};
+      p.run = r; p.nthr = p.n = (int)(hi - lo);
+      p.x0 = reservoir ? lo - ghost : (lo < 0 ? lo + n : lo);
+      p.st_lo = (int)(s0 - lo); p.st_hi = (int)(s1 - lo);
+      pieces->push_back(p);
+    }
+  }
+  return true;
+}
+
+// Tiling of the one-site-per-thread kernel: NT threads per block, k steps per launch (k
+// also bounds the halos; lattices that all fit a block need none and run kwhole steps per
+// launch), spread: one piece per block instead of packed blocks.  us: the estimated time
+// of a step, in microseconds.
+struct BlockedTiling {
+  int NT = 0, k = 0;
+  bool spread = false;
+  double us = 1e300;
+};
+
+// The cheapest tiling by a model of a step's time, fitted to GB300 timings of single
+// lattices of 256 to 2^20 sites and of the 4096-lattice ensemble:
+//   t0 + t1 w + launch / k,
+// w the warps an SM has to step (at least one per scheduler), t0 + 4 t1 the latency of a
+// step with one warp per scheduler (D1Q7: FP64 0.65 us, FP32 0.10 us), t1 the issue time
+// of a warp, launch the time between two launches' work.  More steps per launch mean fewer
+// launches and wider halos, which cost warps; smaller blocks spread a small workload over
+// more SMs.  Two blocks per SM (NT = 384 in FP64) step 12 % slower than three.  The
+// lattices of a large batch are sampled.
+inline BlockedTiling choose_blocked(const std::vector<int64_t>& Ns, bool reservoir, int Q, bool f64, int sms,
+                                    int kwhole) {
+  const int C = (Q - 1) / 2;
+  const double scale = Q == 7 ? 1.0 : 0.7;
+  const double t0 = scale * (f64 ? 0.27 : 0.07), t1 = scale * (f64 ? 0.095 : 0.0075), launch = 1.6;
+  const size_t stride = (Ns.size() + 127) / 128;
+  BlockedTiling best;
+  for (int NT : {64, 96, 128, 192, 256, 384, 512}) {
+    if (f64 && NT > 384) break;
+    for (int k : {4, 6, 8, 12, 16, 24, 32, 48}) {
+      const int64_t h = (int64_t)C * k, room = NT - 2 * h;
+      if (room <= 0) break;
+      bool whole = true;
+      double pieces = 0.0, small = 0.0;  // stretches and whole lattices; the latter's threads
+      int64_t widest = 0;
+      for (size_t r = 0; r < Ns.size(); r += stride) {
+        const int64_t n = Ns[r] + (reservoir ? 2 * C : 0);
+        if (n <= NT) {
+          pieces += 1.0;
+          small += (double)std::max<int64_t>(n, NT / kBlockedPieces) / (0.93 * NT);
+          widest = std::max(widest, n);
+        } else {
+          const int64_t nseg = (n + room - 1) / room;
+          whole = false;
+          pieces += (double)nseg;
+          small += (double)nseg;
+          widest = std::max(widest, (n + nseg - 1) / nseg + 2 * h);
+        }
+      }
+      pieces *= (double)stride;
+      const double blocks = std::max(1.0, small * (double)stride);
+      BlockedTiling b;
+      b.NT = NT;
+      b.k = whole ? kwhole : k;
+      b.spread = pieces <= (double)sms;
+      double w;  // warps per SM
+      if (b.spread) {
+        w = (double)((widest + 31) / 32);
+      } else {
+        const double per = blocks / sms;  // blocks per SM, whole blocks while few
+        w = (per < 3.0 ? std::ceil(per) : per + 0.5) * NT / 32.0;
+        if (f64 && NT > 256) w *= 1.12;
+      }
+      b.us = t0 + t1 * std::max(w, 4.0) + launch / b.k;
+      if (b.us < best.us) best = b;
+      if (whole) break;
+    }
+  }
+  return best;
 }
 
 // Indices 0..n-1 in decreasing order of k (k >= 0), equal keys in index order: the
@@ -306,6 +414,32 @@ inline void pack_blocks(std::vector<Piece>& pieces, int NT, Bins* blocks) {
   blocks->cap = NT;
   for (int i : by_threads_desc(pieces))
     if (!blocks->first_fit(pieces, i)) blocks->open(pieces, i);
+}
+
+// Bundles of the one-site-per-thread kernel: each stretch of a longer lattice has a block of
+// its own (stretches of a lattice are equally long and fill most of it); whole lattices
+// too when spread, else packed first fit after them.
+inline void blocked_bundles(const std::vector<Piece>& pieces, int NT, bool spread, std::vector<Piece>* ordered,
+                            std::vector<int2>* bundles) {
+  ordered->clear();
+  bundles->clear();
+  ordered->reserve(pieces.size());
+  std::vector<Piece> whole;
+  for (const Piece& p : pieces) {
+    if (!spread && p.st_lo == 0 && p.st_hi == p.n) {
+      whole.push_back(p);
+    } else {
+      bundles->push_back(int2{(int)ordered->size(), 1});
+      ordered->push_back(p);
+    }
+  }
+  Bins bins;
+  pack_blocks(whole, NT, &bins);
+  std::vector<Piece> packed;
+  std::vector<int2> more;
+  bins.emit(whole, &packed, &more);
+  for (int2 b : more) bundles->push_back(int2{b.x + (int)ordered->size(), b.y});
+  ordered->insert(ordered->end(), packed.begin(), packed.end());
 }
 
 }  // namespace plan
