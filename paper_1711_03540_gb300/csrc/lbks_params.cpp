@@ -5,6 +5,7 @@
 #include <cstring>
 
 #include "../../include/lb_ks.h"
+#include "lbks_growth.h"
 
 namespace {
 
@@ -144,7 +145,75 @@ double max_abs_eigenvalue(int Q, const double* a, double tau, double kappa) {
   return best;
 }
 
+// Whether every root of the same polynomial lies strictly inside |lambda| = 1 / inv: the
+// Schur-Cohn recursion on the polynomial scaled to the unit disc, about 100 complex
+// multiplications against the root iteration's tens of thousands.  The coefficients: u_j
+// times the quotient of prod_k (lambda - r d_k) by its factor j, by synthetic division.
+// False also when it is too close to call in floating point (a reflection coefficient within
+// 1e-11 of the unit circle; the rounding errors here are below 1e-13).
+bool inside(int Q, const double* a, double tau, double kappa, double inv) {
+  struct C {
+    double x, y;
+  };
+  auto mul = [](C p, C q) { return C{p.x * q.x - p.y * q.y, p.x * q.y + p.y * q.x}; };
+  const double r = 1.0 - 1.0 / tau, w = 1.0 / tau;
+  const C e{std::cos(kappa), -std::sin(kappa)}, e2 = mul(e, e), e3 = mul(e2, e);
+  const C d[7] = {{1.0, 0.0}, e, {e.x, -e.y}, e2, {e2.x, -e2.y}, e3, {e3.x, -e3.y}};
+  C p[8] = {{1.0, 0.0}}, c[8];
+  for (int j = 0; j < Q; ++j)
+    for (int k = j + 1; k >= 1; --k) {
+      const C t = mul(d[j], p[k - 1]);
+      p[k].x = (k <= j ? p[k].x : 0.0) - r * t.x;
+      p[k].y = (k <= j ? p[k].y : 0.0) - r * t.y;
+    }
+  for (int k = 0; k <= Q; ++k) c[k] = p[k];
+  for (int j = 0; j < Q; ++j) {
+    const C u{w * a[j] * d[j].x, w * a[j] * d[j].y};
+    C q = p[0];
+    for (int m = 0; m < Q; ++m) {
+      const C t = mul(u, q), n = mul(d[j], q);
+      c[m + 1].x -= t.x;
+      c[m + 1].y -= t.y;
+      q = C{p[m + 1].x + r * n.x, p[m + 1].y + r * n.y};
+    }
+  }
+  double s = 1.0;
+  for (int k = 1; k <= Q; ++k) {
+    s *= inv;
+    c[k].x *= s;
+    c[k].y *= s;
+  }
+  for (int n = Q; n >= 1; --n) {
+    const C g = c[n];
+    const double m = 1.0 - (g.x * g.x + g.y * g.y);
+    if (!(m > 1e-11)) return false;
+    C b[8];
+    for (int k = 1; k < n; ++k) {
+      const C t = mul(g, C{c[n - k].x, -c[n - k].y});
+      b[k] = C{(c[k].x - t.x) / m, (c[k].y - t.y) / m};
+    }
+    for (int k = 1; k < n; ++k) c[k] = b[k];
+  }
+  return true;
+}
+
 }  // namespace
+
+namespace lbks {
+
+bool growth_exceeds(int scheme, double dx, double dt, double tau, int dm_variant, int nk, double limit) {
+  double A[7], B[7];
+  if (lb_ks_params(scheme, dx, dt, tau, dm_variant, A, B, nullptr) != LB_KS_OK) return false;
+  const double inv = std::exp(-limit * dt);
+  for (int k = 1; k <= nk; ++k) {
+    const double kappa = M_PI * k / nk;
+    if (!inside(scheme, A, tau, kappa, inv) && std::log(max_abs_eigenvalue(scheme, A, tau, kappa)) / dt > limit)
+      return true;
+  }
+  return false;
+}
+
+}  // namespace lbks
 
 extern "C" int lb_ks_max_growth(int scheme, double dx, double dt, double tau, int dm_variant, double rho_bar, int nk,
                                 double* growth) {
