@@ -338,23 +338,13 @@ cudaError_t prepared(int kind, int Q, int prec, int S, int NT, int* out) {
   return cudaSuccess;
 }
 
-// Plan of the blocked kernel (one site per thread): LB_KS_OK, 1 if the plan is not the
-// blocked kernel's (`always` = false and the register-resident kernel is estimated
-// faster), or an error.
-int setup_blocked(lb_ks* h, bool always) {
-  int dev = 0, sms = 0;
-  LBKS_CUDA(h, cudaGetDevice(&dev), "cudaGetDevice");
-  LBKS_CUDA(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute");
+// Plan of the blocked kernel (one site per thread), if its step is estimated to take less
+// than `than` microseconds: LB_KS_OK, 1 if not, or an error.
+int setup_blocked(lb_ks* h, int sms, double than) {
   const int R = h->opts.recentre_every;
   const BlockedTiling b =
       choose_blocked(h->N, h->reservoir, h->Q, h->prec == kF64, sms, R > 0 ? std::min(R, 1000) : 1000);
-  if (b.NT == 0) return 1;
-  // FP32: a step of the register-resident kernel takes 0.88 us with its 5120-site blocks at
-  // most one per SM (0.47 us with one warp per scheduler), more in proportion beyond that
-  if (!always && h->prec != kF64) {
-    const double fill = (double)h->total_sites / (5120.0 * sms);
-    if (b.us > (h->Q == 7 ? 0.88 : 0.62) * std::max(1.0, 1.1 * fill)) return 1;
-  }
+  if (b.NT == 0 || b.us >= than) return 1;
   std::vector<Piece> pieces;
   if (!plan_blocked(h->N, h->reservoir, h->cmax, b.NT, b.k, &pieces)) return 1;
   int bps = 0;
@@ -378,12 +368,17 @@ int setup_blocked(lb_ks* h, bool always) {
   return LB_KS_OK;
 }
 
-// Whether the blocked kernel may run a periodic handle: no tiling asked for, and a storage
-// that is not rounded at launch edges (scaled FP16 is).
-bool blocked_eligible(const lb_ks* h) {
+// Whether the plan of an LB handle is chosen by size: no tiling asked for.
+bool free_tiling(const lb_ks* h) {
   const lb_ks_opts& o = h->opts;
-  return h->nplanes != 1 && h->prec != kF16S && !o.sites_per_thread && !o.threads_per_block && !o.steps_per_launch &&
-         !o.cluster_size;
+  return h->nplanes != 1 && !o.sites_per_thread && !o.threads_per_block && !o.steps_per_launch && !o.cluster_size;
+}
+
+int sm_count(lb_ks* h, int* sms) {
+  int dev = 0;
+  LBKS_CUDA(h, cudaGetDevice(&dev), "cudaGetDevice");
+  LBKS_CUDA(h, cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute");
+  return LB_KS_OK;
 }
 
 // Resident kernel plan.  Whole lattices (rings) run k_ring steps per launch; lattices
@@ -397,33 +392,49 @@ bool blocked_eligible(const lb_ks* h) {
 // the same time; or (merge = 1, or by default when the pairs hold more threads than the
 // single blocks) the single-block bundles go two to a pair on the pair lane's queue.
 // S_force / NT_force / cl_force > 0 pin the tiling and kx_force >= 0 the exchange
-// interval (0: no halves) for autotuner trials; lane_weight is the cost of a pair or
+// interval (0: no halves) for autotuner trials.  Without a tiling from the caller or the
+// tuner, FP64 storage takes the blocked kernel (one site per thread), FP32 that or the
+// register-resident tiling estimated faster (choose_blocked, choose_resident), scaled FP16
+// the latter (its results depend on the steps per launch, which only the resident
+// kernel's whole lattices keep).  lane_weight is the cost of a pair or
 // segment bundle relative to a single-block ring bundle, used to split the blocks.
 int setup_resident(lb_ks* h, bool required, int S_force = 0, int NT_force = 0, double lane_weight = 1.25,
                    int cl_force = 0, int merge = -1, int kx_force = -1) {
   const bool col = h->nplanes == 1;  // the tau = 1 collapse's resident kernel
   h->blocked = false;
-  if (S_force == 1 || (S_force == 0 && blocked_eligible(h))) {
-    const int rc = setup_blocked(h, S_force == 1);
-    if (rc <= 0 || S_force == 1) return rc;
+  int sms = 0, rc;
+  if ((rc = sm_count(h, &sms))) return rc;
+  const int R = h->opts.recentre_every;
+  ResidentTiling fixed;  // S = 0: the first tiling below that holds the lattices
+  if (S_force == 0 && free_tiling(h)) {
+    if (h->prec != kF64)
+      fixed = choose_resident(h->N, h->Q, h->prec == kF16S, sms, R > 0 ? std::min(R, 1000) : 1000,
+                              [&](int S, int NT) { return resident_smem(h->Q, h->prec, S, NT); });
+    // (FP32: beyond 3000 sites an SM the register-resident kernel is always the faster one)
+    const bool may = h->prec == kF64 || (h->prec == kF32 && h->total_sites <= 3000LL * sms);
+    if (may && (rc = setup_blocked(h, sms, h->prec == kF64 ? 1e300 : 0.95 * fixed.us)) <= 0) return rc;
   }
   auto supported = [&](int S, int NT) {
     return col ? collapse_resident_supported(h->Q, h->prec, S, NT) : resident_supported(h->Q, h->prec, S, NT);
   };
   std::vector<int> cand;
+  if (fixed.S) cand.push_back(fixed.S);
   if (S_force) cand.push_back(S_force);
   else if (h->opts.sites_per_thread) cand.push_back(h->opts.sites_per_thread);
   else if (col) cand = h->prec == kF64 ? std::vector<int>{16, 8} : std::vector<int>{32, 16, 8};
   else if (h->prec == kF64) cand = {8, 6, 4};
-  else cand = {20, 18, 12, 8, 16, 6, 4};
-  const int R = h->opts.recentre_every;
-  for (int S : cand) {
+  else cand.insert(cand.end(), {20, 18, 12, 8, 16, 6, 4});
+  for (size_t c = 0; c < cand.size(); ++c) {
+    const int S = cand[c];
+    const bool chosen = fixed.S && c == 0;
     const int NT = NT_force ? NT_force
+                   : chosen ? fixed.NT
                             : (h->opts.threads_per_block ? h->opts.threads_per_block
                                                          : (col ? 256 : default_threads(h->prec, S)));
     if (!supported(S, NT)) continue;
     const int kring = h->opts.steps_per_launch ? h->opts.steps_per_launch : (R > 0 ? std::min(R, 1000) : 1000);
     int kseg = h->opts.steps_per_launch ? h->opts.steps_per_launch
+               : chosen && fixed.kseg    ? fixed.kseg
                                         : std::max(1, (int)((int64_t)NT * S / (20 * h->cmax)));
     kseg = std::min(kseg, kring);
     // default: cluster pairs when some lattice needs more than one block and fits two
@@ -434,7 +445,7 @@ int setup_resident(lb_ks* h, bool required, int S_force = 0, int NT_force = 0, d
     const int kx = cl == 2 ? (kx_force >= 0 ? kx_force : kPairSteps) : 0;
     if (!plan_pieces(h->N, h->cmax, S, NT, cl * NT, kseg, kx, &rings, &segs)) continue;
     Bins blocks, pairs, segbins;
-    pack_rings(rings, NT, &blocks, &pairs);
+    pack_rings(rings, NT, &blocks, &pairs, chosen && fixed.spread);
     // default: one queue of pair work groups when the pairs hold most of the threads
     int pair_thr = 0, block_thr = 0;
     for (size_t b = 0; b < pairs.used.size(); ++b) pair_thr += pairs.used0[b] + pairs.used[b] - NT;
@@ -456,11 +467,7 @@ int setup_resident(lb_ks* h, bool required, int S_force = 0, int NT_force = 0, d
       e = prepared(2, h->Q, h->prec, S, NT, &max_clusters);
       if (e != cudaSuccess || max_clusters < 1) { cudaGetLastError(); continue; }
     }
-    int dev = 0, sms = 0;
-    LBKS_CUDA(h, cudaGetDevice(&dev), "cudaGetDevice");
-    LBKS_CUDA(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute");
     const int slots = bps * sms;  // resident blocks
-    int rc;
     h->nlanes = 0;
     if (!blocks.used.empty()) {
       if ((rc = upload_lane(h, &h->lanes[h->nlanes++], rings, blocks, 1, kring, false, 1.0))) return rc;
@@ -677,7 +684,7 @@ int autotune_resident(lb_ks* h) {
   std::vector<Cand> cands;
   std::vector<std::pair<int, int>> tilings;
   const bool col = h->nplanes == 1;  // the tau = 1 collapse's resident kernel
-  if (blocked_eligible(h)) cands.push_back({1, 0, 1.0, 1, 0, 0});  // one site per thread
+  if (free_tiling(h)) cands.push_back({0, 0, 1.25, 0, -1, -1});  // the choice by size
   if (h->opts.sites_per_thread) {
     tilings.push_back({h->opts.sites_per_thread, h->opts.threads_per_block});
   } else if (col) {
@@ -1033,7 +1040,8 @@ int create_body(lb_ks*& h, lb_ks_t** out, int scheme, int32_t nruns, const int64
     }
   } else if (reservoir) {
     kern = LB_KS_KERNEL_PLAIN;
-    if (h->prec != kF16S && (rc = setup_blocked(h, true)) < 0) return bail(rc);
+    int sms = 0;
+    if ((rc = sm_count(h, &sms)) || (h->prec != kF16S && (rc = setup_blocked(h, sms, 1e300)) < 0)) return bail(rc);
   } else if (kern == LB_KS_KERNEL_AUTO || kern == LB_KS_KERNEL_RESIDENT) {
     rc = setup_resident(h, kern == LB_KS_KERNEL_RESIDENT);
     if (rc < 0) return bail(rc);

@@ -2,6 +2,7 @@
 // Not part of the public ABI (that is include/lb_ks.h).
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -130,6 +131,7 @@ struct ResidentLaunch {
   bool one = false;                // blocked kernel: every bundle holds one piece
 };
 bool resident_supported(int Q, int storage, int S, int NT);
+size_t resident_smem(int Q, int storage, int S, int NT);  // dynamic shared memory of a block
 cudaError_t resident_prepare(int Q, int storage, int S, int NT, int* blocks_per_sm);
 // The tau = 1 collapse (one stored plane).
 int collapse_tile_sites();

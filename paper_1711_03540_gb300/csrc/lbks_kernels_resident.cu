@@ -36,6 +36,11 @@ bool resident_supported(int Q, int storage, int S, int NT) {
   return NT >= 32 && NT <= maxt && NT % 32 == 0;
 }
 
+size_t resident_smem(int Q, int storage, int S, int NT) {
+  LBKS_RESIDENT_DISPATCH(return (smem_bytes_t<Qc, STc, Sc>(NT)));
+  return 0;
+}
+
 cudaError_t resident_prepare(int Q, int storage, int S, int NT, int* blocks_per_sm) {
   if (!resident_supported(Q, storage, S, NT)) return cudaErrorInvalidValue;
   LBKS_RESIDENT_DISPATCH(return (prepare_t<Qc, STc, Sc>(NT, blocks_per_sm)));

@@ -357,11 +357,142 @@ inline std::vector<int> by_threads_desc(const std::vector<Piece>& pieces) {
   return stable_desc(nthr);
 }
 
+// Time of a step of the register-resident kernel (D1Q7, microseconds), S sites per thread
+// and q warps on each of an SM's schedulers, measured on single lattices and on uniform
+// batches that fill the device; 0: not a tiling that choose_resident considers.
+inline double resident_step_us(int S, int q) {
+  const auto at = [q](double first, double more) { return first + more * (q - 1); };
+  switch (S) {
+    case 20: return at(0.48, 0.375);
+    case 18: return at(0.385, 0.335);
+    case 16: return at(0.345, 0.315);
+    case 8: return at(0.285, 0.175);
+    case 6: return at(0.26, 0.127);
+    case 4: return at(0.235, 0.10);
+    default: return 0.0;
+  }
+}
+
+// Tiling of the register-resident kernel for FP32 and scaled FP16 storage.  spread: one
+// lattice per block instead of packed ones; kseg: steps per launch of segments (0: the
+// fixed rule's); us: the estimated time of a step.
+struct ResidentTiling {
+  int S = 0, NT = 0, kseg = 0;
+  bool spread = false;
+  double us = 1e300;
+};
+
+// The estimate for one tiling of which `bps` blocks fit an SM: blocks run in rounds of
+// sms bps, each as long as a full SM's step, so a batch of 1.7 rounds takes as long as
+// one of 2, and smaller blocks that need 2 shorter rounds are faster; a batch of less
+// than a round runs as fast as its fullest SM.  Segments (FP32 alone: scaled FP16 rounds at
+// launch edges, so its launches stay as they are): each launch adds `edge` microseconds per
+// round for loads and stores (measured on a 2^24-site lattice), and halos of c_max kseg
+// sites; kseg is the cheapest, or kfix.
+inline ResidentTiling rate_resident(const std::vector<int64_t>& Ns, int Q, int S, int NT, int bps, int sms, bool f16,
+                                    int kmax, bool may_spread, int kfix = 0) {
+  const double edge = S == 18 ? 14.5 : 20.0;
+  constexpr double kLaunchUs = 3.0, kFill = 0.97, kHalfCost = 1.05, kRingCost = 1.4, kRingUs = 0.4;
+  const int C = (Q - 1) / 2, h = C * kPairStepsMax;
+  const double scale = Q == 7 ? 1.0 : 0.7;
+  ResidentTiling t;
+  t.S = S;
+  t.NT = NT;
+  const size_t stride = (Ns.size() + 255) / 256;
+  double pieces = 0.0, blocks = 0.0;
+  int64_t widest = 0;
+  std::vector<int64_t> cut;
+  bool pairs = false, ring = false;
+  for (size_t r = 0; r < Ns.size(); r += stride) {
+    const int64_t v = (Ns[r] + S - 1) / S, half = ((Ns[r] + 1) / 2 + 2 * h + S - 1) / S + 1;
+    if (v <= NT) {
+      pieces += 1.0;
+      blocks += (double)v / (kFill * NT);
+      widest = std::max(widest, v);
+    } else if (half <= NT) {
+      pieces += 2.0;
+      blocks += kHalfCost * 2.0 * (double)half / (kFill * NT);
+      widest = NT;
+      pairs = true;
+    } else if (v <= 2 * NT) {  // one ring across a pair waits on the other block every step
+      if (!kfix) return t;     // (the fixed tiling's estimate is still wanted)
+      ring = true;
+      pieces += 1.0;
+      blocks += kRingCost * (double)v / (kFill * NT);
+      widest = NT;
+      pairs = true;
+    } else {
+      cut.push_back(Ns[r]);
+    }
+  }
+  pieces *= (double)stride;
+  blocks *= (double)stride;
+  const double slots = (double)sms * bps;
+  const auto warps = [&](double per_sm, int64_t threads) {  // per scheduler
+    return (int)std::ceil(per_sm * (double)((threads + 31) / 32) / 4.0 - 1e-9);
+  };
+  double us = ring ? kRingUs : 0.0;
+  if (pieces > 0.0) {
+    t.spread = may_spread && !pairs && cut.empty() && pieces <= slots;
+    if (t.spread) {
+      us = scale * resident_step_us(S, warps(std::ceil(pieces / sms), widest));
+    } else {
+      const double rounds = std::ceil(blocks / slots);
+      us = scale * rounds * resident_step_us(S, warps(std::min<double>(bps, std::ceil(blocks / sms)), NT));
+    }
+  }
+  if (!cut.empty()) {
+    if (f16) return t;
+    const double full = scale * resident_step_us(S, warps(bps, NT));
+    double best = 1e300;
+    for (int k = kfix ? kfix : 16; k <= std::min(kmax, 192); k += 8) {
+      const int64_t room = (int64_t)NT * S - 2LL * C * k - 2 * S;
+      if (room <= 0) break;
+      double n = 0.0;
+      for (int64_t N : cut) n += (double)((N + room - 1) / room);
+      const double rounds = std::ceil(n * (double)stride / slots);
+      const double c = rounds * (full + edge / k) + kLaunchUs / k;
+      if (c < best) { best = c; t.kseg = k; }
+      if (kfix) break;
+    }
+    us += best;
+  }
+  t.us = us;
+  return t;
+}
+
+// The register-resident tiling of a batch.  The fixed tiling (20 sites x 256 threads,
+// lattices packed) stays unless another is estimated at least 8 % faster, about the
+// estimate's error on large ensembles; S = 0: it stays.  us is the chosen one's estimate.
+// smem(S, NT): shared memory of a block.
+template <typename F>
+ResidentTiling choose_resident(const std::vector<int64_t>& Ns, int Q, bool f16, int sms, int kmax, F smem) {
+  const auto fit = [&](int S, int NT) {  // blocks per SM by registers (255 a thread above 8 sites) and shared memory
+    const int threads = S <= 8 ? 512 : 256;
+    return std::max(1, std::min(threads / NT, (int)(228 * 1024 / (smem(S, NT) + 1024))));
+  };
+  const ResidentTiling fixed =
+      rate_resident(Ns, Q, 20, 256, 1, sms, f16, kmax, false, std::min(kmax, 5120 / (10 * (Q - 1))));
+  ResidentTiling best;
+  best.us = fixed.us;
+  int64_t sites = 0, longest = 0;
+  for (int64_t n : Ns) { sites += n; longest = std::max(longest, n); }
+  if (longest <= 10240 && sites > 6LL * 5120 * sms) return best;  // more than six rounds: nothing to gain by 8 %
+  if (f16 && fixed.us > 1e290) return best;  // segments: their launches round
+  for (const auto& c : {std::pair<int, int>{20, 256}, {18, 256}, {16, 256}, {18, 128}, {16, 128}, {8, 512}, {8, 256},
+                        {6, 512}, {6, 256}, {4, 512}, {4, 256}, {4, 128}}) {
+    const ResidentTiling t = rate_resident(Ns, Q, c.first, c.second, fit(c.first, c.second), sms, f16, kmax, true);
+    if (t.us < 0.92 * fixed.us && t.us < best.us) best = t;
+  }
+  return best;
+}
+
 // First-fit decreasing packing of whole lattices: a lattice held as two halves opens a
 // cluster pair (one half at the start of each block), one longer than one block (more
 // than NT threads) opens a pair as a ring across both blocks; the others fill the
 // pairs' spare threads first, then blocks of NT threads.
-inline void pack_rings(std::vector<Piece>& pieces, int NT, Bins* blocks, Bins* pairs) {
+// (spread: these open a block each).
+inline void pack_rings(std::vector<Piece>& pieces, int NT, Bins* blocks, Bins* pairs, bool spread = false) {
   blocks->cap = NT;
   pairs->cap = 2 * NT;
   pairs->pair = true;
@@ -377,7 +508,7 @@ inline void pack_rings(std::vector<Piece>& pieces, int NT, Bins* blocks, Bins* p
     if (pieces[i].nthr > NT) {
       pieces[i].t0 = 0;
       pairs->add({i}, NT, pieces[i].nthr);
-    } else if (!pairs->first_fit(pieces, i) && !blocks->first_fit(pieces, i)) {
+    } else if (spread || (!pairs->first_fit(pieces, i) && !blocks->first_fit(pieces, i))) {
       blocks->open(pieces, i);
     }
   }

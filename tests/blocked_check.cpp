@@ -77,6 +77,27 @@ int main() {
               return 1;
             }
           }
+  // the register-resident choice holds every lattice whole that the fixed tiling does, and
+  // leaves scaled FP16 batches with segments alone (their launches round)
+  for (int Q : {5, 7})
+    for (bool f16 : {false, true})
+      for (int i = 0; i < 300; ++i) {
+        std::vector<int64_t> Ns(1 + rng() % (i % 3 ? 40u : 1500u));
+        const unsigned span = 20u << (rng() % 10u);
+        for (auto& n : Ns) n = 7 + (int)(rng() % span);
+        const ResidentTiling t = choose_resident(Ns, Q, f16, 152, 500, [](int S, int NT) { return (size_t)S * NT * 40; });
+        if (t.S == 0) continue;
+        int64_t longest = 0;
+        for (int64_t n : Ns) longest = std::max(longest, n);
+        std::vector<Piece> rings, segs, rings20, segs20;
+        const int C = (Q - 1) / 2, cl = longest > t.S * t.NT && longest <= 2 * t.S * t.NT ? 2 : 1;
+        const bool held = plan_pieces(Ns, C, t.S, t.NT, cl * t.NT, t.kseg ? t.kseg : 8, cl == 2 ? 32 : 0, &rings, &segs);
+        plan_pieces(Ns, C, 20, 256, longest > 5120 ? 512 : 256, 85, 32, &rings20, &segs20);
+        if (!held || (f16 && (!segs20.empty() || !segs.empty()))) {
+          std::printf("resident tiling S %d NT %d for %zu lattices up to %lld\n", t.S, t.NT, Ns.size(), (long long)longest);
+          return 1;
+        }
+      }
   std::printf("ok\n");
   return 0;
 }

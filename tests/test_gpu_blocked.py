@@ -90,3 +90,20 @@ def test_reservoir_ends_match_oracle(lb, Q, runs):
         outs.append(out)
     assert np.max(np.abs(outs[0] - ref)) <= 1e-12 * np.abs(ref).max()
     np.testing.assert_array_equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("prec", [1, 2])
+@pytest.mark.parametrize("nruns,nmin,nmax", [(1, 1000, 1000), (4, 500, 2700), (24, 256, 8192), (60, 100, 600),
+                                             (238, 164, 549), (354, 548, 1770), (1024, 64, 256), (2500, 100, 700),
+                                             (1024, 220, 4000), (3, 9000, 11000)])
+def test_tiling_chosen_by_size_equals_the_fixed_one(lb, prec, nruns, nmin, nmax):
+    """FP32 and scaled FP16 (rounded at launch edges, which the choice must not move): the
+    default plan's results are those of 20 sites x 256 threads, bitwise."""
+    rng = np.random.default_rng(71)
+    Ns = np.round(np.exp(rng.uniform(np.log(nmin), np.log(nmax), nruns))).astype(np.int64)
+    r0 = np.concatenate([0.02 * rng.standard_normal(n) for n in Ns])
+    kw = dict(precision=prec, recentre_every=60)
+    a, _ = _run(lb, 7, Ns, r0, (130,), **kw)
+    b, d = _run(lb, 7, Ns, r0, (130,), sites_per_thread=20, threads_per_block=256, **kw)
+    assert d["sites_per_thread"] == 20
+    np.testing.assert_array_equal(a, b)
