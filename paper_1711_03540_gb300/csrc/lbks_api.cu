@@ -342,14 +342,16 @@ cudaError_t prepared(int kind, int Q, int prec, int S, int NT, int* out) {
 // than `than` microseconds: LB_KS_OK, 1 if not, or an error.
 int setup_blocked(lb_ks* h, int sms, double than) {
   const int R = h->opts.recentre_every;
-  const BlockedTiling b =
-      choose_blocked(h->N, h->reservoir, h->Q, h->prec == kF64, sms, R > 0 ? std::min(R, 1000) : 1000);
+  const BlockedTiling b = choose_blocked(h->N, h->reservoir, h->Q, blocked_cost(h->Q, h->prec == kF64, h->nplanes == 1),
+                                         sms, R > 0 ? std::min(R, 1000) : 1000);
   if (b.NT == 0 || b.us >= than) return 1;
   std::vector<Piece> pieces;
   if (!plan_blocked(h->N, h->reservoir, h->cmax, b.NT, b.k, &pieces)) return 1;
-  int bps = 0;
-  cudaError_t e = prepared(h->reservoir ? 4 : 3, h->Q, h->prec, 1, b.NT, &bps);
-  if (e != cudaSuccess || bps < 1) { cudaGetLastError(); return 1; }
+  if (h->nplanes > 1) {
+    int bps = 0;
+    cudaError_t e = prepared(h->reservoir ? 4 : 3, h->Q, h->prec, 1, b.NT, &bps);
+    if (e != cudaSuccess || bps < 1) { cudaGetLastError(); return 1; }
+  }
   std::vector<Piece> ordered;
   std::vector<int2> bundles;
   blocked_bundles(pieces, b.NT, b.spread, &ordered, &bundles);
@@ -371,7 +373,7 @@ int setup_blocked(lb_ks* h, int sms, double than) {
 // Whether the plan of an LB handle is chosen by size: no tiling asked for.
 bool free_tiling(const lb_ks* h) {
   const lb_ks_opts& o = h->opts;
-  return h->nplanes != 1 && !o.sites_per_thread && !o.threads_per_block && !o.steps_per_launch && !o.cluster_size;
+  return !o.sites_per_thread && !o.threads_per_block && !o.steps_per_launch && !o.cluster_size;
 }
 
 int sm_count(lb_ks* h, int* sms) {
@@ -406,7 +408,14 @@ int setup_resident(lb_ks* h, bool required, int S_force = 0, int NT_force = 0, d
   if ((rc = sm_count(h, &sms))) return rc;
   const int R = h->opts.recentre_every;
   ResidentTiling fixed;  // S = 0: the first tiling below that holds the lattices
-  if (S_force == 0 && free_tiling(h)) {
+  if (col && S_force == 0 && free_tiling(h)) {
+    // FP32: a step of the register-resident collapse takes about 1 us a round of its
+    // 8192-site blocks; FP64: 28 us a round of 4096 sites, bound by the FP64 pipe as the
+    // blocked collapse is, which spreads over the SMs and cuts no lattice into few blocks
+    const double us = (h->Q == 7 ? 1.0 : 0.75) * std::max(1.0, 1.03 * (double)h->total_sites / (8192.0 * sms));
+    if ((rc = setup_blocked(h, sms, h->prec == kF64 ? 1e300 : 0.95 * us)) <= 0) return rc;
+  }
+  if (!col && S_force == 0 && free_tiling(h)) {
     if (h->prec != kF64)
       fixed = choose_resident(h->N, h->Q, h->prec == kF16S, sms, R > 0 ? std::min(R, 1000) : 1000,
                               [&](int S, int NT) { return resident_smem(h->Q, h->prec, S, NT); });
@@ -1037,6 +1046,9 @@ int create_body(lb_ks*& h, lb_ks_t** out, int scheme, int32_t nruns, const int64
       rc = setup_resident(h, false);
       if (rc < 0) return bail(rc);
       h->collapse_resident = rc == 0;
+    } else if (reservoir && o.steps_per_launch != 1) {
+      int sms = 0;
+      if ((rc = sm_count(h, &sms)) || (rc = setup_blocked(h, sms, 1e300)) < 0) return bail(rc);
     }
   } else if (reservoir) {
     kern = LB_KS_KERNEL_PLAIN;

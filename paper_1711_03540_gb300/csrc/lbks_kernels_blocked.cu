@@ -28,6 +28,7 @@
 // 4096-lattice FP64 ensemble 615 -> 219 us per step, 4.3e10 site-updates/s (256 threads, 4
 // steps per launch; bound by the integer pipe, 54 % busy, and the conversions, 56 %), 122
 // front lattices 9.3 -> 2.3 us per step, 24 FP32 lattices 0.87 -> 0.37 us per step.
+#include "lbks_collapse.cuh"
 #include "lbks_device.cuh"
 #include "lbks_plan.h"
 
@@ -130,6 +131,67 @@ __global__ void __launch_bounds__(BlockedCfg<Q, ST>::kMaxThreads, BlockedCfg<Q, 
   }
 }
 
+// The tau = 1 collapse in the same form: one value per thread, its 2 c_max neighbours read
+// from the exchange area each step (with the guard columns for wrapping ends).  FP64
+// storage, FP32 batches too small for the register-resident collapse, and reservoir ends
+// (the fixed nodes keep their values, put in both parities once).  FP64 is bound by the
+// FP64 pipe, so what counts is to use every SM's: one 4096-site lattice 25 -> 1.0 us per
+// step, 24 lattices 25 -> 3.9, the 4096-lattice ensemble 442 -> 418; FP32, 24 lattices: 1.02
+// -> 0.34 us, one lattice 0.57 -> 0.20 (300 lattices: 1.03 either way, so larger batches
+// stay register-resident).
+template <int C, int ST, bool RES, bool ONE>
+__global__ void __launch_bounds__(512, 2)
+    blocked_collapse_kernel(Arena src, Arena dst, const RunDesc* __restrict__ runs, const Piece* __restrict__ pieces,
+                            const int2* __restrict__ bundles, int ksteps) {
+  using T = typename StorageType<ST>::type;
+  using CT = typename StorageType<ST>::compute;
+  constexpr int XS = 512 + 2 * C * kBlockedPieces;
+  __shared__ CT ex[2][XS];
+  const int t = threadIdx.x;
+  int p = blockIdx.x, q = 0;
+  if constexpr (!ONE) {
+    const int2 bd = bundles[blockIdx.x];
+    p = bd.x;
+    for (int u = 1; u < bd.y; ++u)
+      if (t >= pieces[bd.x + u].t0) q = u;
+    p += q;
+  }
+  const Piece pc = pieces[p];
+  const int n = pc.n, j = t - pc.t0;
+  const bool active = j < n;
+  wait_prior_grid();
+  const RunDesc& d = runs[pc.run];
+  int x = (int)pc.x0 + j;
+  bool fixed = false;
+  if constexpr (RES) fixed = x <= 0 || x >= (int)d.N - 1;
+  else if (x >= (int)d.N) x -= (int)d.N;
+  CT v = CT(0);
+  if (active) v = static_cast<CT>(static_cast<const T*>(src.f)[d.off + x]);
+  const CollapseCoef<CT, C> k = load_collapse_coef<CT, C>(d);
+  CT* const own = &ex[0][t + C * (2 * q + 1)];
+  const bool last = j >= n - C, first = j < C;  // these also enter at the other end
+  for (int s = 0; s < ksteps; ++s) {
+    CT* const xs = own + (s & 1) * XS;
+    if (active && (!RES || !fixed || s < 2)) {
+      *xs = v;
+      if (last) xs[-n] = v;
+      if (first) xs[n] = v;
+    }
+    __syncthreads();
+    if (active && !fixed) {
+      CT dl[C + 1], dr[C + 1];
+      dl[0] = dr[0] = CT(0);
+#pragma unroll
+      for (int c = 1; c <= C; ++c) {
+        dl[c] = xs[-c];
+        dr[c] = xs[c];
+      }
+      v = collapse_site<CT, C>(v, dl, dr, k);
+    }
+  }
+  if (active && !fixed && j >= pc.st_lo && j < pc.st_hi) static_cast<T*>(dst.f)[d.off + x] = static_cast<T>(v);
+}
+
 template <int Q, int ST, bool RES>
 cudaError_t prepare_t(int NT, int* blocks_per_sm) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, blocked_step_kernel<Q, ST, RES, false>, NT, 0);
@@ -137,8 +199,21 @@ cudaError_t prepare_t(int NT, int* blocks_per_sm) {
 
 template <int Q, int ST, bool RES>
 cudaError_t launch_t(const ResidentLaunch& L, cudaStream_t s) {
-  return launch_early(L.one ? blocked_step_kernel<Q, ST, RES, true> : blocked_step_kernel<Q, ST, RES, false>, L.nbundles,
-                      L.NT, 0, s, L.src, L.dst, L.runs, L.pieces, L.bundles, L.ksteps);
+  if (L.one)
+    return launch_early(blocked_step_kernel<Q, ST, RES, true>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs, L.pieces,
+                        L.bundles, L.ksteps);
+  return launch_early(blocked_step_kernel<Q, ST, RES, false>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs, L.pieces,
+                      L.bundles, L.ksteps);
+}
+
+template <int Q, int ST, bool RES>
+cudaError_t launch_collapse_t(const ResidentLaunch& L, cudaStream_t s) {
+  constexpr int C = cmax_of(Q);
+  if (L.one)
+    return launch_early(blocked_collapse_kernel<C, ST, RES, true>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs, L.pieces,
+                        L.bundles, L.ksteps);
+  return launch_early(blocked_collapse_kernel<C, ST, RES, false>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs, L.pieces,
+                      L.bundles, L.ksteps);
 }
 
 #define LBKS_BLOCKED_DISPATCH(OP)                                                    \
@@ -152,7 +227,7 @@ cudaError_t launch_t(const ResidentLaunch& L, cudaStream_t s) {
 }  // namespace
 
 bool blocked_supported(int Q, int storage, int NT) {
-  return (Q == 5 || Q == 7) && (storage == kF64 || storage == kF32) && NT >= 32 && NT <= (storage == kF64 ? 384 : 512) && NT % 32 == 0;
+  return (Q == 5 || Q == 7) && (storage == kF64 || storage == kF32) && NT >= 32 && NT <= 512 && NT % 32 == 0;
 }
 
 cudaError_t blocked_prepare(int Q, int storage, int NT, bool reservoir, int* blocks_per_sm) {
@@ -166,6 +241,12 @@ cudaError_t launch_blocked(const ResidentLaunch& L, bool reservoir, cudaStream_t
   const int Q = L.Q, storage = L.storage;
   if (!blocked_supported(Q, storage, L.NT)) return cudaErrorInvalidValue;
   if (L.nbundles == 0) return cudaSuccess;
+  if (L.collapse) {
+    if (reservoir) LBKS_BLOCKED_DISPATCH(return (launch_collapse_t<Qc, STc, true>(L, s)));
+    else LBKS_BLOCKED_DISPATCH(return (launch_collapse_t<Qc, STc, false>(L, s)));
+    return cudaErrorInvalidValue;
+  }
+  if (L.NT > (storage == kF64 ? 384 : 512)) return cudaErrorInvalidValue;
   if (reservoir) LBKS_BLOCKED_DISPATCH(return (launch_t<Qc, STc, true>(L, s)));
   else LBKS_BLOCKED_DISPATCH(return (launch_t<Qc, STc, false>(L, s)));
   return cudaErrorInvalidValue;

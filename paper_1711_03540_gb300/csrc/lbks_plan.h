@@ -175,24 +175,37 @@ struct BlockedTiling {
   double us = 1e300;
 };
 
-// The cheapest tiling by a model of a step's time, fitted to GB300 timings of single
-// lattices of 256 to 2^20 sites and of the 4096-lattice ensemble:
-//   t0 + t1 w + launch / k,
-// w the warps an SM has to step (at least one per scheduler), t0 + 4 t1 the latency of a
-// step with one warp per scheduler (D1Q7: FP64 0.65 us, FP32 0.10 us), t1 the issue time
-// of a warp, launch the time between two launches' work.  More steps per launch mean fewer
-// launches and wider halos, which cost warps; smaller blocks spread a small workload over
-// more SMs.  Two blocks per SM (NT = 384 in FP64) step 12 % slower than three.  The
-// lattices of a large batch are sampled.
-inline BlockedTiling choose_blocked(const std::vector<int64_t>& Ns, bool reservoir, int Q, bool f64, int sms,
-                                    int kwhole) {
+// A model of a step's time in microseconds, fitted to GB300 timings of single lattices of
+// 256 to 2^20 sites and of the 4096-lattice ensembles:
+//   t0 + t1 max(w, wmin) + launch / k,
+// w the warps an SM has to step, t1 the issue time of one, wmin one per scheduler (t0 + 4 t1
+// is then the latency of a step: D1Q7 FP64 0.65 us, FP32 0.10 us; the FP64 collapse, in
+// FP64 arithmetic, is bound by the FP64 pipe the schedulers share), launch the time
+// between two launches' work.
+struct BlockedCost {
+  double t0, t1, launch;
+  int wmin, max_threads;
+};
+inline BlockedCost blocked_cost(int Q, bool f64, bool collapse) {
+  BlockedCost c = collapse ? (f64 ? BlockedCost{0.10, 0.21, 3.2, 1, 512} : BlockedCost{0.10, 0.007, 3.2, 4, 512})
+                           : (f64 ? BlockedCost{0.27, 0.095, 1.6, 4, 384} : BlockedCost{0.07, 0.0075, 1.6, 4, 512});
+  if (Q == 5) {
+    c.t0 *= 0.7;
+    c.t1 *= 0.7;
+  }
+  return c;
+}
+
+// The cheapest tiling.  More steps per launch mean fewer launches and wider halos, which
+// cost warps; smaller blocks spread a small workload over more SMs.  Two blocks per SM
+// (NT = 384 in FP64) step 12 % slower than three.  The lattices of a large batch are sampled.
+inline BlockedTiling choose_blocked(const std::vector<int64_t>& Ns, bool reservoir, int Q, const BlockedCost& cost,
+                                    int sms, int kwhole) {
   const int C = (Q - 1) / 2;
-  const double scale = Q == 7 ? 1.0 : 0.7;
-  const double t0 = scale * (f64 ? 0.27 : 0.07), t1 = scale * (f64 ? 0.095 : 0.0075), launch = 1.6;
   const size_t stride = (Ns.size() + 127) / 128;
   BlockedTiling best;
   for (int NT : {64, 96, 128, 192, 256, 384, 512}) {
-    if (f64 && NT > 384) break;
+    if (NT > cost.max_threads) break;
     for (int k : {4, 6, 8, 12, 16, 24, 32, 48}) {
       const int64_t h = (int64_t)C * k, room = NT - 2 * h;
       if (room <= 0) break;
@@ -225,9 +238,9 @@ inline BlockedTiling choose_blocked(const std::vector<int64_t>& Ns, bool reservo
       } else {
         const double per = blocks / sms;  // blocks per SM, whole blocks while few
         w = (per < 3.0 ? std::ceil(per) : per + 0.5) * NT / 32.0;
-        if (f64 && NT > 256) w *= 1.12;
+        if (cost.max_threads == 384 && NT > 256) w *= 1.12;
       }
-      b.us = t0 + t1 * std::max(w, 4.0) + launch / b.k;
+      b.us = cost.t0 + cost.t1 * std::max<double>(w, cost.wmin) + cost.launch / b.k;
       if (b.us < best.us) best = b;
       if (whole) break;
     }

@@ -64,14 +64,15 @@ int main() {
   // the chosen tilings hold what they are chosen for
   for (int Q : {5, 7})
     for (bool f64 : {false, true})
+     for (bool col : {false, true})
       for (bool res : {false, true})
         for (int64_t n : {7, 60, 400, 513, 4096, 100001, 1 << 24})
           for (int runs : {1, 40, 3000}) {
             if (n * runs > (1 << 24)) continue;
             const std::vector<int64_t> Ns((size_t)runs, n);
-            const BlockedTiling b = choose_blocked(Ns, res, Q, f64, 152, 500);
+            const BlockedTiling b = choose_blocked(Ns, res, Q, blocked_cost(Q, f64, col), 152, 500);
             std::vector<Piece> pieces;
-            if (b.NT < 32 || b.NT > (f64 ? 384 : 512) || b.NT % 32 || b.k < 1 ||
+            if (b.NT < 32 || b.NT > (f64 && !col ? 384 : 512) || b.NT % 32 || b.k < 1 ||
                 !plan_blocked(Ns, res, (Q - 1) / 2, b.NT, b.k, &pieces)) {
               std::printf("tiling NT %d k %d for %d x %lld\n", b.NT, b.k, runs, (long long)n);
               return 1;

@@ -107,3 +107,49 @@ def test_tiling_chosen_by_size_equals_the_fixed_one(lb, prec, nruns, nmin, nmax)
     b, d = _run(lb, 7, Ns, r0, (130,), sites_per_thread=20, threads_per_block=256, **kw)
     assert d["sites_per_thread"] == 20
     np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("Q", [5, 7])
+@pytest.mark.parametrize("which", SIZES)
+def test_blocked_collapse_equals_streaming_bitwise(lb, prec, Q, which):
+    """The tau = 1 collapse, one value per thread, against one step per launch."""
+    Ns, r0 = _batch(Q if which == "Q" else which, Q)
+    k, outs = len(Ns), []
+    for spl, calls in ((0, (1, 53, 100)), (1, (154,))):
+        h = lb.lb_ks_batch_init(Q, Ns, Ns * 0.2, np.full(k, 5e-5), np.ones(k), r0, lb.lb_ks_default_opts(
+            kernel=lb.KERNEL_COLLAPSE, precision=prec, recentre_every=70 if prec else 0, steps_per_launch=spl))
+        try:
+            for n in calls:
+                lb.lb_ks_step(h, n)
+            out = np.empty(r0.size)
+            lb.lb_ks_rho(h, out)
+            spt = lb.lb_ks_describe(h)["sites_per_thread"]
+        finally:
+            lb.lb_ks_free(h)
+        assert spt == (0 if spl else 1)
+        outs.append(out)
+    np.testing.assert_array_equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("Q", [5, 7])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_blocked_collapse_reservoir_ends(lb, Q, prec):
+    """Reservoir ends on the collapse: many steps per launch against one."""
+    alphas = [0.4, 0.2, 0.1]
+    Ns = np.array([front.nodes(a).size for a in alphas], dtype=np.int64)
+    r0 = np.concatenate([front.rho_exact(front.nodes(a), 0.0) for a in alphas])
+    outs = []
+    for spl in (0, 1):
+        h = lb.lb_ks_batch_init_reservoir(Q, Ns, np.full(3, 60.0), np.full(3, 2e-6), np.ones(3), r0,
+                                          np.full(3, front.RHO_LEFT), np.full(3, front.RHO_RIGHT), lb.lb_ks_default_opts(
+                                              kernel=lb.KERNEL_COLLAPSE, precision=prec, steps_per_launch=spl))
+        try:
+            for n in (2, 131):
+                lb.lb_ks_step(h, n)
+            out = np.empty(r0.size)
+            lb.lb_ks_rho(h, out)
+        finally:
+            lb.lb_ks_free(h)
+        outs.append(out)
+    np.testing.assert_array_equal(outs[0], outs[1])
