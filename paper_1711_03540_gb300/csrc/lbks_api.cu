@@ -781,9 +781,9 @@ int check_flags(lb_ks* h) {
 // Linear stability check (lb_ks_max_growth, nk = 128, about rho = 0) of every distinct
 // (dx, dt, tau) when a batch has at most 64 of them; a run whose growth rate exceeds
 // 1.05 x 1/4 leaves a warning in last_error (the handle is still created).  Each distinct
-// set is decided once, by growth_exceeds: the roots at all 128 phases took 3.6 ms a set
+// set is decided once, by growth_above: the roots at all 128 phases took 3.6 ms a set
 // (11 ms of creating three small lattices; 21 s for 4096 lattices that share one), the
-// decision takes about 0.03 ms; the rate itself is computed for the first unstable run alone.
+// decision takes about 0.01 ms; the rate itself is computed for the first unstable run alone.
 void warn_if_linearly_unstable(lb_ks* h, const double* L, const double* dt, const double* tau) {
   constexpr double kLimit = 1.05 * 0.25;
   struct Set {
@@ -803,14 +803,14 @@ void warn_if_linearly_unstable(lb_ks* h, const double* L, const double* dt, cons
     }
     of[r] = (int)s;
   }
-  for (Set& s : sets) s.unstable = growth_exceeds(h->Q, s.key[0], s.key[1], s.key[2], h->opts.dm_variant, 128, kLimit);
+  for (Set& s : sets)
+    s.unstable = growth_above(h->Q, s.key[0], s.key[1], s.key[2], h->opts.dm_variant, 128, kLimit, true) > kLimit;
   int bad = 0, first = -1;
   for (int32_t r = 0; r < h->nruns; ++r)
     if (sets[of[r]].unstable && bad++ == 0) first = r;
   if (!bad) return;
   const auto& k = sets[of[first]].key;
-  double worst = 0.0;
-  lb_ks_max_growth(h->Q, k[0], k[1], k[2], h->opts.dm_variant, 0.0, 128, &worst);
+  const double worst = growth_above(h->Q, k[0], k[1], k[2], h->opts.dm_variant, 128, kLimit, false);
   h->err = "warning: " + std::to_string(bad) + " run(s) linearly unstable (run " + std::to_string(first) +
            ": growth rate " + std::to_string(worst) + " per unit time > 1.05 x 1/4)";
 }

@@ -145,54 +145,59 @@ double max_abs_eigenvalue(int Q, const double* a, double tau, double kappa) {
   return best;
 }
 
-// Whether every root of the same polynomial lies strictly inside |lambda| = 1 / inv: the
-// Schur-Cohn recursion on the polynomial scaled to the unit disc, about 100 complex
-// multiplications against the root iteration's tens of thousands.  The coefficients: u_j
-// times the quotient of prod_k (lambda - r d_k) by its factor j, by synthetic division.
+// Whether every root of the same polynomial lies strictly inside |lambda| = 1 / inv, for
+// even a (a_{+c} = a_{-c}, as A is): the Schur-Cohn recursion on the polynomial scaled to
+// the unit disc, some hundred multiplications against the root iteration's tens of
+// thousands.  The speeds +-c pair into real quadratics q_c = lambda^2 - 2 r cos(c kappa)
+// lambda + r^2, so that
+//   p = (lambda - r - w a_0) prod_c q_c - (lambda - r) sum_c 2 w a_c (cos(c kappa) lambda - r) prod_{c' != c} q_c'.
 // False also when it is too close to call in floating point (a reflection coefficient within
-// 1e-11 of the unit circle; the rounding errors here are below 1e-13).
-bool inside(int Q, const double* a, double tau, double kappa, double inv) {
-  struct C {
-    double x, y;
-  };
-  auto mul = [](C p, C q) { return C{p.x * q.x - p.y * q.y, p.x * q.y + p.y * q.x}; };
-  const double r = 1.0 - 1.0 / tau, w = 1.0 / tau;
-  const C e{std::cos(kappa), -std::sin(kappa)}, e2 = mul(e, e), e3 = mul(e2, e);
-  const C d[7] = {{1.0, 0.0}, e, {e.x, -e.y}, e2, {e2.x, -e2.y}, e3, {e3.x, -e3.y}};
-  C p[8] = {{1.0, 0.0}}, c[8];
-  for (int j = 0; j < Q; ++j)
-    for (int k = j + 1; k >= 1; --k) {
-      const C t = mul(d[j], p[k - 1]);
-      p[k].x = (k <= j ? p[k].x : 0.0) - r * t.x;
-      p[k].y = (k <= j ? p[k].y : 0.0) - r * t.y;
+// 1e-11 of 1; the rounding errors here are below 1e-13).
+template <int Q>
+bool inside(const double* a, double tau, double kappa, double inv) {
+  constexpr int P = (Q - 1) / 2;
+  const double r = 1.0 - 1.0 / tau, w = 1.0 / tau, c1 = std::cos(kappa);
+  const double cs[3] = {c1, 2.0 * c1 * c1 - 1.0, c1 * (4.0 * c1 * c1 - 3.0)};
+  // all = prod q_c and part = sum_c 2 w a_c (cos lambda - r) prod_{c' != c} q_c', highest power first
+  double all[8] = {1.0}, part[8] = {};
+  for (int c = 0; c < P; ++c) {
+    const double q1 = -2.0 * r * cs[c], q2 = r * r, f = 2.0 * w * a[2 * c + 1];
+    double na[8] = {}, np[8] = {};
+    for (int k = 0; k <= 2 * c; ++k) {  // (part has degree 2 c - 1, all 2 c)
+      np[k] += part[k];
+      np[k + 1] += q1 * part[k];
+      np[k + 2] += q2 * part[k];
+      na[k] += all[k];
+      na[k + 1] += q1 * all[k];
+      na[k + 2] += q2 * all[k];
     }
-  for (int k = 0; k <= Q; ++k) c[k] = p[k];
-  for (int j = 0; j < Q; ++j) {
-    const C u{w * a[j] * d[j].x, w * a[j] * d[j].y};
-    C q = p[0];
-    for (int m = 0; m < Q; ++m) {
-      const C t = mul(u, q), n = mul(d[j], q);
-      c[m + 1].x -= t.x;
-      c[m + 1].y -= t.y;
-      q = C{p[m + 1].x + r * n.x, p[m + 1].y + r * n.y};
+    // both as polynomials of degree 2 c + 2: part's leading coefficient is 0
+    for (int k = 0; k <= 2 * c; ++k) {
+      np[k + 1] += f * cs[c] * all[k];
+      np[k + 2] -= f * r * all[k];
     }
+    for (int k = 0; k <= 2 * c + 2; ++k) {
+      all[k] = na[k];
+      part[k] = np[k];
+    }
+  }
+  double p[8] = {};
+  for (int k = 0; k < Q; ++k) {
+    p[k] += all[k] - part[k];
+    p[k + 1] += r * part[k] - (r + w * a[0]) * all[k];
   }
   double s = 1.0;
-  for (int k = 1; k <= Q; ++k) {
-    s *= inv;
-    c[k].x *= s;
-    c[k].y *= s;
-  }
+  for (int k = 1; k <= Q; ++k) p[k] *= (s *= inv);
   for (int n = Q; n >= 1; --n) {
-    const C g = c[n];
-    const double m = 1.0 - (g.x * g.x + g.y * g.y);
-    if (!(m > 1e-11)) return false;
-    C b[8];
-    for (int k = 1; k < n; ++k) {
-      const C t = mul(g, C{c[n - k].x, -c[n - k].y});
-      b[k] = C{(c[k].x - t.x) / m, (c[k].y - t.y) / m};
+    // (undivided: each step scales what is left by p[0]^2 - p[n]^2)
+    const double f = p[0], g = p[n], m = f * f - g * g;
+    if (!(m > 1e-11 * f * f)) return false;
+    p[0] = m;
+    for (int k = 1, l = n - 1; k <= l; ++k, --l) {
+      const double x = p[k], y = p[l];
+      p[k] = f * x - g * y;
+      p[l] = f * y - g * x;
     }
-    for (int k = 1; k < n; ++k) c[k] = b[k];
   }
   return true;
 }
@@ -201,16 +206,20 @@ bool inside(int Q, const double* a, double tau, double kappa, double inv) {
 
 namespace lbks {
 
-bool growth_exceeds(int scheme, double dx, double dt, double tau, int dm_variant, int nk, double limit) {
+double growth_above(int scheme, double dx, double dt, double tau, int dm_variant, int nk, double limit, bool first) {
   double A[7], B[7];
-  if (lb_ks_params(scheme, dx, dt, tau, dm_variant, A, B, nullptr) != LB_KS_OK) return false;
-  const double inv = std::exp(-limit * dt);
+  if (lb_ks_params(scheme, dx, dt, tau, dm_variant, A, B, nullptr) != LB_KS_OK) return limit;
+  double best = limit, inv = std::exp(-best * dt);
   for (int k = 1; k <= nk; ++k) {
     const double kappa = M_PI * k / nk;
-    if (!inside(scheme, A, tau, kappa, inv) && std::log(max_abs_eigenvalue(scheme, A, tau, kappa)) / dt > limit)
-      return true;
+    if (scheme == LB_KS_D1Q5 ? inside<5>(A, tau, kappa, inv) : inside<7>(A, tau, kappa, inv)) continue;
+    const double g = std::log(max_abs_eigenvalue(scheme, A, tau, kappa)) / dt;
+    if (!(g > best)) continue;
+    if (first) return g;
+    best = g;
+    inv = std::exp(-best * dt);
   }
-  return false;
+  return best;
 }
 
 }  // namespace lbks

@@ -17,7 +17,9 @@ int main() {
     double g = 0.0;
     if (lb_ks_max_growth(Q, dx, dt, tau, variant, 0.0, 128, &g) != LB_KS_OK) return 1;
     for (double limit : {1.05 * 0.25, g + 1e-3 * std::fabs(g) + 1e-6, g - 1e-3 * std::fabs(g) - 1e-6})
-      if (lbks::growth_exceeds(Q, dx, dt, tau, variant, 128, limit) != (g > limit)) {
+      if ((lbks::growth_above(Q, dx, dt, tau, variant, 128, limit, true) > limit) != (g > limit) ||
+          std::fabs(lbks::growth_above(Q, dx, dt, tau, variant, 128, limit, false) - std::fmax(g, limit)) >
+              1e-9 * std::fabs(g) + 1e-10 / dt) {
         std::printf("D1Q%d dx %g dt %g tau %g variant %d: growth %g limit %g\n", Q, dx, dt, tau, variant, g, limit);
         return 1;
       }

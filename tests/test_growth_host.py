@@ -1,5 +1,5 @@
 """The constructors' linear stability decision (csrc/lbks_growth.h) equals lb_ks_max_growth's
-rate compared with the limit, over random spacings, time steps, relaxation times and
+rate compared with the limit, and the rate reported above it that rate, over random spacings, time steps, relaxation times and
 readings of both schemes, at the library's limit and just above and below the rate."""
 import os
 import subprocess
