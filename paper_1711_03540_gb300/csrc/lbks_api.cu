@@ -315,7 +315,7 @@ int upload_lane(lb_ks* h, Lane* L, const std::vector<Piece>& pieces, const Bins&
 
 // The kernels' launch preparation (dynamic shared memory opt-in, resident blocks per SM
 // or clusters at once), done once per device, kind (0 resident, 1 collapse, 2 cluster
-// pairs, 3 and 4 one site per thread, periodic and reservoir), scheme, storage and tiling: the attribute set by it stays with the function.
+// pairs), scheme, storage and tiling: the attribute set by it stays with the function.
 cudaError_t prepared(int kind, int Q, int prec, int S, int NT, int* out) {
   static std::mutex mu;
   static std::map<std::array<int, 6>, int> done;
@@ -329,8 +329,7 @@ cudaError_t prepared(int kind, int Q, int prec, int S, int NT, int* out) {
     int v = 0;
     e = kind == 0 ? resident_prepare(Q, prec, S, NT, &v)
         : kind == 1 ? collapse_resident_prepare(Q, prec, S, NT, &v)
-        : kind == 2 ? resident_cluster_prepare(Q, prec, S, NT, &v)
-                    : blocked_prepare(Q, prec, NT, kind == 4, &v);
+                    : resident_cluster_prepare(Q, prec, S, NT, &v);
     if (e != cudaSuccess) return e;  // not kept: the caller clears the error and tries another tiling
     it = done.emplace(key, v).first;
   }
@@ -347,11 +346,6 @@ int setup_blocked(lb_ks* h, int sms, double than) {
   if (b.NT == 0 || b.us >= than) return 1;
   std::vector<Piece> pieces;
   if (!plan_blocked(h->N, h->reservoir, h->cmax, b.NT, b.k, &pieces)) return 1;
-  if (h->nplanes > 1) {
-    int bps = 0;
-    cudaError_t e = prepared(h->reservoir ? 4 : 3, h->Q, h->prec, 1, b.NT, &bps);
-    if (e != cudaSuccess || bps < 1) { cudaGetLastError(); return 1; }
-  }
   std::vector<Piece> ordered;
   std::vector<int2> bundles;
   blocked_bundles(pieces, b.NT, b.spread, &ordered, &bundles);

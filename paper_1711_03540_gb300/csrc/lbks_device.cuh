@@ -132,12 +132,11 @@ __device__ __forceinline__ int64_t wrap_site(int64_t x, int64_t N) {
 // scheduled while this one runs instead of after it.  Every thread first waits until
 // the grid before it in the stream (the previous step, which reads this step's
 // destination and writes its source) has completed and its writes are visible; only
-// then does it touch global memory and let the next grid be scheduled.  In a grid
-// launched without the attribute both instructions return at once.
-__device__ __forceinline__ void wait_prior_grid() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+// then does it touch the populations and let the next grid be scheduled (the
+// many-step kernels only near their end).  In a grid launched without the attribute both
+// instructions return at once.
+__device__ __forceinline__ void wait_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Launch with programmatic stream serialisation allowed (for kernels that start with
 // wait_prior_grid): the grid may be scheduled before the kernel ahead of it in the

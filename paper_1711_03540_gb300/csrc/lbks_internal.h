@@ -151,7 +151,6 @@ cudaError_t launch_resident(const ResidentLaunch& L, cudaStream_t s);
 // One site per thread, ksteps steps per launch (lbks_kernels_blocked.cu): bundles of
 // pieces, one block each (ResidentLaunch::nbundles blocks, no queue).
 bool blocked_supported(int Q, int storage, int NT);
-cudaError_t blocked_prepare(int Q, int storage, int NT, bool reservoir, int* blocks_per_sm);
 cudaError_t launch_blocked(const ResidentLaunch& L, bool reservoir, cudaStream_t s);
 
 // Diagnostic micro-benchmark of the FMA pipes (flop/s), used by the benchmark

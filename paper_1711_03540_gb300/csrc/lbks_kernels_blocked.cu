@@ -38,28 +38,34 @@ namespace {
 
 using plan::kBlockedPieces;
 
-template <int Q, int ST> struct BlockedCfg {
-  static constexpr int kMaxThreads = ST == kF64 ? 384 : 512;
-  // blocks of kMaxThreads an SM holds: sets the register budget (80 and 64)
-  static constexpr int kMinBlocks = 2;
+// The next launch's blocks may be scheduled from this many steps before the end.  Earlier,
+// they fill the SMs' free slots around the running blocks, unevenly (an SM with fewer of
+// these gets more of those, up to five instead of four on a batch of 3.6 blocks an SM:
+// 3.4 instead of 2.4 us per step); at the last step, a small batch waits for the launch.
+constexpr int kNextGrid = 2;
+
+// NTM: the most threads a block of this instance has.
+template <int Q, int ST, int NTM> struct BlockedCfg {
+  // blocks of NTM an SM holds: sets the register budget (FP64 80, FP32 64)
+  static constexpr int kMinBlocks = (ST == kF64 ? 768 : 1024) / NTM;
   // Row of the exchange area, a compile-time stride: a column per thread.  FP64: and, for
   // each piece, c_max on either side of its own, where the threads at the piece's other end
   // put the values that wrap, so that every access is one address plus an immediate and no
   // registers are held for the neighbours.  FP32 has the registers: the six neighbours'
   // columns are computed once, which takes fewer instructions per step.
   static constexpr bool kGuard = ST == kF64;
-  static constexpr int kXS = kMaxThreads + (kGuard ? 2 * cmax_of(Q) * kBlockedPieces : 0);
+  static constexpr int kXS = NTM + (kGuard ? 2 * cmax_of(Q) * kBlockedPieces : 0);
 };
 
 // ONE: every bundle holds one piece.
-template <int Q, int ST, bool RES, bool ONE>
-__global__ void __launch_bounds__(BlockedCfg<Q, ST>::kMaxThreads, BlockedCfg<Q, ST>::kMinBlocks)
+template <int Q, int ST, int NTM, bool RES, bool ONE>
+__global__ void __launch_bounds__(NTM, (BlockedCfg<Q, ST, NTM>::kMinBlocks))
     blocked_step_kernel(Arena src, Arena dst, const RunDesc* __restrict__ runs, const Piece* __restrict__ pieces,
                         const int2* __restrict__ bundles, int ksteps) {
   using T = typename StorageType<ST>::type;
   using CT = typename StorageType<ST>::compute;
-  constexpr int C = cmax_of(Q), XS = BlockedCfg<Q, ST>::kXS;
-  constexpr bool kGuard = BlockedCfg<Q, ST>::kGuard;
+  constexpr int C = cmax_of(Q), XS = BlockedCfg<Q, ST, NTM>::kXS;
+  constexpr bool kGuard = BlockedCfg<Q, ST, NTM>::kGuard;
   __shared__ CT ex[2][Q - 1][XS];  // [step parity][plane i - 1]
   // (the pieces are written once, before any launch)
   const int t = threadIdx.x;
@@ -95,6 +101,7 @@ __global__ void __launch_bounds__(BlockedCfg<Q, ST>::kMaxThreads, BlockedCfg<Q, 
     from[i] = (i & 1) ? (j >= c ? -c : n - c) : (j + c < n ? c : c - n);
   }
   for (int s = 0; s < ksteps; ++s) {
+    if (s == ksteps - kNextGrid || (s == 0 && ksteps < kNextGrid)) allow_next_grid();
     CT* const xs = own + (s & 1) * (Q - 1) * XS;
     if (active && (!RES || !fixed || s < 3)) {
       collide<Q>(g, k);
@@ -171,6 +178,7 @@ __global__ void __launch_bounds__(512, 2)
   CT* const own = &ex[0][t + C * (2 * q + 1)];
   const bool last = j >= n - C, first = j < C;  // these also enter at the other end
   for (int s = 0; s < ksteps; ++s) {
+    if (s == ksteps - kNextGrid || (s == 0 && ksteps < kNextGrid)) allow_next_grid();
     CT* const xs = own + (s & 1) * XS;
     if (active && (!RES || !fixed || s < 2)) {
       *xs = v;
@@ -192,18 +200,26 @@ __global__ void __launch_bounds__(512, 2)
   if (active && !fixed && j >= pc.st_lo && j < pc.st_hi) static_cast<T*>(dst.f)[d.off + x] = static_cast<T>(v);
 }
 
-template <int Q, int ST, bool RES>
-cudaError_t prepare_t(int NT, int* blocks_per_sm) {
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, blocked_step_kernel<Q, ST, RES, false>, NT, 0);
+template <int Q, int ST, bool RES, int NTM>
+cudaError_t launch_n(const ResidentLaunch& L, cudaStream_t s) {
+  if (L.one)
+    return launch_early(blocked_step_kernel<Q, ST, NTM, RES, true>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs, L.pieces,
+                        L.bundles, L.ksteps);
+  return launch_early(blocked_step_kernel<Q, ST, NTM, RES, false>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs, L.pieces,
+                      L.bundles, L.ksteps);
 }
 
+// The exchange area is sized by the instance, and FP64's would otherwise bound the blocks
+// per SM: 128 threads (21 KB), 256 (34 KB) and 384 (46 KB).
 template <int Q, int ST, bool RES>
 cudaError_t launch_t(const ResidentLaunch& L, cudaStream_t s) {
-  if (L.one)
-    return launch_early(blocked_step_kernel<Q, ST, RES, true>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs, L.pieces,
-                        L.bundles, L.ksteps);
-  return launch_early(blocked_step_kernel<Q, ST, RES, false>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs, L.pieces,
-                      L.bundles, L.ksteps);
+  if constexpr (ST == kF64) {
+    if (L.NT <= 128) return launch_n<Q, ST, RES, 128>(L, s);
+    if (L.NT <= 256) return launch_n<Q, ST, RES, 256>(L, s);
+    return launch_n<Q, ST, RES, 384>(L, s);
+  } else {
+    return launch_n<Q, ST, RES, 512>(L, s);
+  }
 }
 
 template <int Q, int ST, bool RES>
@@ -228,13 +244,6 @@ cudaError_t launch_collapse_t(const ResidentLaunch& L, cudaStream_t s) {
 
 bool blocked_supported(int Q, int storage, int NT) {
   return (Q == 5 || Q == 7) && (storage == kF64 || storage == kF32) && NT >= 32 && NT <= 512 && NT % 32 == 0;
-}
-
-cudaError_t blocked_prepare(int Q, int storage, int NT, bool reservoir, int* blocks_per_sm) {
-  if (!blocked_supported(Q, storage, NT)) return cudaErrorInvalidValue;
-  if (reservoir) LBKS_BLOCKED_DISPATCH(return (prepare_t<Qc, STc, true>(NT, blocks_per_sm)));
-  else LBKS_BLOCKED_DISPATCH(return (prepare_t<Qc, STc, false>(NT, blocks_per_sm)));
-  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_blocked(const ResidentLaunch& L, bool reservoir, cudaStream_t s) {

@@ -42,6 +42,7 @@ __global__ void __launch_bounds__(kCollapseThreads) collapse_step_kernel(Arena s
   using CT = typename StorageType<ST>::compute;
   __shared__ CT buf[kCollapseTile + 2 * C];
   wait_prior_grid();
+  allow_next_grid();
   const Tile tl = tiles[blockIdx.x];
   const RunDesc& d = runs[tl.run];
   const T* fs = static_cast<const T*>(src.f) + d.off;

@@ -159,6 +159,7 @@ __global__ void __launch_bounds__(kPlainThreads) plain_step_kernel(Arena src, Ar
   using T = typename StorageType<ST>::type;
   using CT = typename StorageType<ST>::compute;
   wait_prior_grid();
+  allow_next_grid();
   const Tile tl = tiles[blockIdx.x];
   if ((int)threadIdx.x >= tl.len) return;
   const RunDesc& d = runs[tl.run];
@@ -198,6 +199,7 @@ __global__ void __launch_bounds__(kPlainThreads) reservoir_step_kernel(Arena src
   using T = typename StorageType<ST>::type;
   using CT = typename StorageType<ST>::compute;
   wait_prior_grid();
+  allow_next_grid();
   const Tile tl = tiles[blockIdx.x];
   if ((int)threadIdx.x >= tl.len) return;
   const RunDesc& d = runs[tl.run];

@@ -123,6 +123,7 @@ __device__ __forceinline__ void stream_step(Arena src, Arena dst, const RunDesc*
   };
 
   wait_prior_grid();
+  allow_next_grid();
   const Tile tl = tiles[blockIdx.x];
   const RunDesc& d = runs[tl.run];
   const Coef<CT, Q> k = load_coef<CT, Q>(d);

@@ -181,7 +181,9 @@ struct BlockedTiling {
 // w the warps an SM has to step, t1 the issue time of one, wmin one per scheduler (t0 + 4 t1
 // is then the latency of a step: D1Q7 FP64 0.65 us, FP32 0.10 us; the FP64 collapse, in
 // FP64 arithmetic, is bound by the FP64 pipe the schedulers share), launch the time
-// between two launches' work.
+// between two launches' work (with several FP64 blocks an SM kMoreLaunch times as long: the
+// last blocks of one launch end apart).
+constexpr double kMoreLaunch = 2.4;
 struct BlockedCost {
   double t0, t1, launch;
   int wmin, max_threads;
@@ -197,8 +199,9 @@ inline BlockedCost blocked_cost(int Q, bool f64, bool collapse) {
 }
 
 // The cheapest tiling.  More steps per launch mean fewer launches and wider halos, which
-// cost warps; smaller blocks spread a small workload over more SMs.  Two blocks per SM
-// (NT = 384 in FP64) step 12 % slower than three.  The lattices of a large batch are sampled.
+// cost warps; smaller blocks spread a small workload over more SMs.  FP64 blocks of more
+// than 128 threads step 8 to 20 % slower on a full device (their warps meet at the barrier
+// and then want the same pipe).  The lattices of a large batch are sampled.
 inline BlockedTiling choose_blocked(const std::vector<int64_t>& Ns, bool reservoir, int Q, const BlockedCost& cost,
                                     int sms, int kwhole) {
   const int C = (Q - 1) / 2;
@@ -206,7 +209,7 @@ inline BlockedTiling choose_blocked(const std::vector<int64_t>& Ns, bool reservo
   BlockedTiling best;
   for (int NT : {64, 96, 128, 192, 256, 384, 512}) {
     if (NT > cost.max_threads) break;
-    for (int k : {4, 6, 8, 12, 16, 24, 32, 48}) {
+    for (int k : {2, 3, 4, 6, 8, 12, 16, 24, 32, 48}) {
       const int64_t h = (int64_t)C * k, room = NT - 2 * h;
       if (room <= 0) break;
       bool whole = true;
@@ -238,9 +241,9 @@ inline BlockedTiling choose_blocked(const std::vector<int64_t>& Ns, bool reservo
       } else {
         const double per = blocks / sms;  // blocks per SM, whole blocks while few
         w = (per < 3.0 ? std::ceil(per) : per + 0.5) * NT / 32.0;
-        if (cost.max_threads == 384 && NT > 256) w *= 1.12;
+        if (cost.max_threads == 384 && NT > 128) w *= NT > 256 ? 1.2 : 1.08;
       }
-      b.us = cost.t0 + cost.t1 * std::max<double>(w, cost.wmin) + cost.launch / b.k;
+      b.us = cost.t0 + cost.t1 * std::max<double>(w, cost.wmin) + cost.launch * (b.spread || cost.max_threads != 384 ? 1.0 : kMoreLaunch) / b.k;
       if (b.us < best.us) best = b;
       if (whole) break;
     }
