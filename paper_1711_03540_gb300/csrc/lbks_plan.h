@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <functional>
 #include <initializer_list>
 #include <utility>
 #include <vector>
@@ -375,8 +376,11 @@ inline std::vector<int> by_threads_desc(const std::vector<Piece>& pieces) {
 
 // Time of a step of the register-resident kernel (D1Q7, microseconds), S sites per thread
 // and q warps on each of an SM's schedulers, measured on single lattices and on uniform
-// batches that fill the device; 0: not a tiling that choose_resident considers.
-inline double resident_step_us(int S, int q) {
+// batches that fill the device; 0: not a tiling that choose_resident considers.  Two blocks
+// of 128 threads overlap one's barrier with the other's step: 14 to 17 % less per site than
+// one of 256 (1.07e12 and 1.08e12 site-updates/s at 18 and 16 sites, 0.92e12 at 20 x 256).
+inline double resident_step_us(int S, int NT, int q) {
+  if (NT == 128 && q == 2 && (S == 18 || S == 16)) return S == 18 ? 0.654 : 0.575;
   const auto at = [q](double first, double more) { return first + more * (q - 1); };
   switch (S) {
     case 20: return at(0.48, 0.375);
@@ -407,59 +411,62 @@ struct ResidentTiling {
 // sites; kseg is the cheapest, or kfix.
 inline ResidentTiling rate_resident(const std::vector<int64_t>& Ns, int Q, int S, int NT, int bps, int sms, bool f16,
                                     int kmax, bool may_spread, int kfix = 0) {
-  const double edge = S == 18 ? 14.5 : 20.0;
-  constexpr double kLaunchUs = 3.0, kFill = 0.97, kHalfCost = 1.05, kRingCost = 1.4, kRingUs = 0.4;
+  const double edge = S == 18 ? 14.5 : 20.0, half_cost = NT < 256 ? 1.2 : 1.05;
+  constexpr double kLaunchUs = 3.0, kRingCost = 1.4, kRingUs = 0.4;
   const int C = (Q - 1) / 2, h = C * kPairStepsMax;
   const double scale = Q == 7 ? 1.0 : 0.7;
   ResidentTiling t;
   t.S = S;
   t.NT = NT;
-  const size_t stride = (Ns.size() + 255) / 256;
-  double pieces = 0.0, blocks = 0.0;
-  int64_t widest = 0;
+  const size_t stride = (Ns.size() + 127) / 128;  // a sample of a large batch
+  std::vector<int> threads;  // of whole lattices and halves
+  int64_t halves = 0, rings = 0;
   std::vector<int64_t> cut;
-  bool pairs = false, ring = false;
   for (size_t r = 0; r < Ns.size(); r += stride) {
     const int64_t v = (Ns[r] + S - 1) / S, half = ((Ns[r] + 1) / 2 + 2 * h + S - 1) / S + 1;
     if (v <= NT) {
-      pieces += 1.0;
-      blocks += (double)v / (kFill * NT);
-      widest = std::max(widest, v);
+      threads.push_back((int)v);
     } else if (half <= NT) {
-      pieces += 2.0;
-      blocks += kHalfCost * 2.0 * (double)half / (kFill * NT);
-      widest = NT;
-      pairs = true;
+      threads.insert(threads.end(), 2, (int)half);
+      halves += 2;
     } else if (v <= 2 * NT) {  // one ring across a pair waits on the other block every step
       if (!kfix) return t;     // (the fixed tiling's estimate is still wanted)
-      ring = true;
-      pieces += 1.0;
-      blocks += kRingCost * (double)v / (kFill * NT);
-      widest = NT;
-      pairs = true;
+      ++rings;
     } else {
       cut.push_back(Ns[r]);
     }
   }
-  pieces *= (double)stride;
-  blocks *= (double)stride;
+  const bool pairs = halves + rings > 0;
+  const double pieces = (double)(threads.size() + rings) * (double)stride;
+  // first fit, largest first: the blocks they fill
+  std::sort(threads.begin(), threads.end(), std::greater<int>());
+  const int64_t widest = pairs ? NT : (threads.empty() ? 0 : threads.front());
+  std::vector<int> room;
+  for (int v : threads) {
+    size_t b = 0;
+    while (b < room.size() && room[b] < v) ++b;
+    if (b == room.size()) room.push_back(NT);
+    room[b] -= v;
+  }
+  const double blocks = ((double)room.size() * (1.0 + (half_cost - 1.0) * (double)halves / std::max<double>(1.0, (double)threads.size())) +
+                         2.0 * kRingCost * (double)rings) * (double)stride;
   const double slots = (double)sms * bps;
   const auto warps = [&](double per_sm, int64_t threads) {  // per scheduler
     return (int)std::ceil(per_sm * (double)((threads + 31) / 32) / 4.0 - 1e-9);
   };
-  double us = ring ? kRingUs : 0.0;
+  double us = rings ? kRingUs : 0.0;
   if (pieces > 0.0) {
     t.spread = may_spread && !pairs && cut.empty() && pieces <= slots;
     if (t.spread) {
-      us = scale * resident_step_us(S, warps(std::ceil(pieces / sms), widest));
+      us = scale * resident_step_us(S, NT, warps(std::ceil(pieces / sms), widest));
     } else {
       const double rounds = std::ceil(blocks / slots);
-      us = scale * rounds * resident_step_us(S, warps(std::min<double>(bps, std::ceil(blocks / sms)), NT));
+      us = scale * rounds * resident_step_us(S, NT, warps(std::min<double>(bps, std::ceil(blocks / sms)), NT));
     }
   }
   if (!cut.empty()) {
     if (f16) return t;
-    const double full = scale * resident_step_us(S, warps(bps, NT));
+    const double full = scale * resident_step_us(S, NT, warps(bps, NT));
     double best = 1e300;
     for (int k = kfix ? kfix : 16; k <= std::min(kmax, 192); k += 8) {
       const int64_t room = (int64_t)NT * S - 2LL * C * k - 2 * S;
@@ -493,7 +500,8 @@ ResidentTiling choose_resident(const std::vector<int64_t>& Ns, int Q, bool f16, 
   best.us = fixed.us;
   int64_t sites = 0, longest = 0;
   for (int64_t n : Ns) { sites += n; longest = std::max(longest, n); }
-  if (longest <= 10240 && sites > 6LL * 5120 * sms) return best;  // more than six rounds: nothing to gain by 8 %
+  // more than six rounds: little to gain from their number, only from two blocks an SM
+  if (longest > 2304 && longest <= 10240 && sites > 6LL * 5120 * sms) return best;
   if (f16 && fixed.us > 1e290) return best;  // segments: their launches round
   for (const auto& c : {std::pair<int, int>{20, 256}, {18, 256}, {16, 256}, {18, 128}, {16, 128}, {8, 512}, {8, 256},
                         {6, 512}, {6, 256}, {4, 512}, {4, 256}, {4, 128}}) {

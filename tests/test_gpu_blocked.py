@@ -62,7 +62,9 @@ def test_blocked_equals_plain_bitwise(lb, prec, Q, which):
     kw = dict(precision=prec, recentre_every=70 if prec else 0)
     a, da = _run(lb, Q, Ns, r0, (1, 53, 100), **kw)
     b, _ = _run(lb, Q, Ns, r0, (154,), kernel=1, **kw)
-    assert da["kernel"] == lb.KERNEL_RESIDENT and da["sites_per_thread"] == 1
+    assert da["kernel"] == lb.KERNEL_RESIDENT
+    if prec == 0 or len(Ns) == 1:  # (FP32 batches: whichever tiling is estimated faster)
+        assert da["sites_per_thread"] == 1
     np.testing.assert_array_equal(a, b)
 
 
