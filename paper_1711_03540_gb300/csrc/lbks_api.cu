@@ -65,6 +65,7 @@ struct Lane {
   bool merged = false;  // cl = 2: single-block bundles run two to a pair work group
   int halves = 0;       // lattices held as two halves
   bool one = false;     // every bundle holds one piece
+  bool spread = false;  // at most one block per SM
   Piece* d_pieces = nullptr;
   int2* d_bundles = nullptr;
   int* d_queue = nullptr;
@@ -357,6 +358,7 @@ int setup_blocked(lb_ks* h, int sms, double than) {
   if ((rc = upload_lane(h, &L, ordered, bundles, 1, b.k, segmented, 1.0))) return rc;
   L.grid = L.nbundles;
   L.one = bundles.size() == pieces.size();
+  L.spread = b.spread && L.nbundles <= sms;
   h->nlanes = 1;
   h->blocked = true;
   h->S = 1;
@@ -528,7 +530,7 @@ int issue_lane(lb_ks* h, const Lane& L, int64_t k, int from, bool in_place, cuda
     if (!h->blocked) LBKS_CUDA(h, cudaMemsetAsync(L.d_queue, 0, sizeof(int), s), "queue reset");
     ResidentLaunch RL{h->Q, h->prec, h->S, h->NT, arena(h, cur), arena(h, dst), h->d_runs,
                       L.d_pieces, L.d_bundles, L.nbundles, L.d_queue, (int)kk, L.grid, L.cl, h->d_flags,
-                      h->nplanes == 1, L.kx, h->link_wait_limit, h->link_withhold_step, L.one};
+                      h->nplanes == 1, L.kx, h->link_wait_limit, h->link_withhold_step, L.one, L.spread};
     LBKS_CUDA(h, h->blocked ? launch_blocked(RL, h->reservoir, s) : launch_resident(RL, s), "resident step");
     *nk += 1;
     cur = dst;

@@ -129,6 +129,7 @@ struct ResidentLaunch {
   uint32_t wait_limit = 1u << 22;  // cl = 2: try_wait rounds before a wait on the other block gives up
   int withhold_step = -1;          // cl = 2, testing aid: block 1 sends nothing across the edge at this step
   bool one = false;                // blocked kernel: every bundle holds one piece
+  bool spread = false;             // ... and there is at most one block per SM
 };
 bool resident_supported(int Q, int storage, int S, int NT);
 size_t resident_smem(int Q, int storage, int S, int NT);  // dynamic shared memory of a block

@@ -46,8 +46,6 @@ constexpr int kNextGrid = 2;
 
 // NTM: the most threads a block of this instance has.
 template <int Q, int ST, int NTM> struct BlockedCfg {
-  // blocks of NTM an SM holds: sets the register budget (FP64 80, FP32 64)
-  static constexpr int kMinBlocks = (ST == kF64 ? 768 : 1024) / NTM;
   // Row of the exchange area, a compile-time stride: a column per thread.  FP64: and, for
   // each piece, c_max on either side of its own, where the threads at the piece's other end
   // put the values that wrap, so that every access is one address plus an immediate and no
@@ -57,9 +55,12 @@ template <int Q, int ST, int NTM> struct BlockedCfg {
   static constexpr int kXS = NTM + (kGuard ? 2 * cmax_of(Q) * kBlockedPieces : 0);
 };
 
-// ONE: every bundle holds one piece.
-template <int Q, int ST, int NTM, bool RES, bool ONE>
-__global__ void __launch_bounds__(NTM, (BlockedCfg<Q, ST, NTM>::kMinBlocks))
+// ONE: every bundle holds one piece.  MINB: blocks an SM has to hold, which sets the
+// register budget: 80 in FP64 (24 warps), 64 in FP32 where SMs are to be filled; FP64 batches
+// of at most a block per SM take what the compiler wants instead (122), which shortens the
+// one warp per scheduler's chain by 4 to 6 %.
+template <int Q, int ST, int NTM, int MINB, bool RES, bool ONE>
+__global__ void __launch_bounds__(NTM, MINB)
     blocked_step_kernel(Arena src, Arena dst, const RunDesc* __restrict__ runs, const Piece* __restrict__ pieces,
                         const int2* __restrict__ bundles, int ksteps) {
   using T = typename StorageType<ST>::type;
@@ -202,11 +203,12 @@ __global__ void __launch_bounds__(512, 2)
 
 template <int Q, int ST, bool RES, int NTM>
 cudaError_t launch_n(const ResidentLaunch& L, cudaStream_t s) {
+  constexpr int MINB = (ST == kF64 ? 768 : 1024) / NTM;
   if (L.one)
-    return launch_early(blocked_step_kernel<Q, ST, NTM, RES, true>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs, L.pieces,
-                        L.bundles, L.ksteps);
-  return launch_early(blocked_step_kernel<Q, ST, NTM, RES, false>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs, L.pieces,
-                      L.bundles, L.ksteps);
+    return launch_early(blocked_step_kernel<Q, ST, NTM, MINB, RES, true>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs,
+                        L.pieces, L.bundles, L.ksteps);
+  return launch_early(blocked_step_kernel<Q, ST, NTM, MINB, RES, false>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs,
+                      L.pieces, L.bundles, L.ksteps);
 }
 
 // The exchange area is sized by the instance, and FP64's would otherwise bound the blocks
@@ -214,6 +216,9 @@ cudaError_t launch_n(const ResidentLaunch& L, cudaStream_t s) {
 template <int Q, int ST, bool RES>
 cudaError_t launch_t(const ResidentLaunch& L, cudaStream_t s) {
   if constexpr (ST == kF64) {
+    if (L.NT <= 128 && L.one && L.spread)
+      return launch_early(blocked_step_kernel<Q, ST, 128, 1, RES, true>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs,
+                          L.pieces, L.bundles, L.ksteps);
     if (L.NT <= 128) return launch_n<Q, ST, RES, 128>(L, s);
     if (L.NT <= 256) return launch_n<Q, ST, RES, 256>(L, s);
     return launch_n<Q, ST, RES, 384>(L, s);
