@@ -98,6 +98,7 @@ using RunTable = std::vector<RunDesc, NoInitAlloc<RunDesc>>;
 struct lb_ks {
   int Q = 0, prec = 0, kernel = 0, cmax = 0;
   int nplanes = 0;         // stored planes: Q, or 1 for the tau = 1 collapse (rho - rhobar)
+  bool zb = false;       // the kernels' instances without the terms that add zero (zero_terms)
   bool blocked = false;  // one site per thread, many steps per launch (one lane, S = 1)
   bool collapse_resident = false;  // tau = 1 collapse on its register-resident kernel (lanes below)
   bool reservoir = false;  // lattices with fixed-value ends instead of periodic ones
@@ -318,20 +319,20 @@ int upload_lane(lb_ks* h, Lane* L, const std::vector<Piece>& pieces, const Bins&
 // The kernels' launch preparation (dynamic shared memory opt-in, resident blocks per SM
 // or clusters at once), done once per device, kind (0 resident, 1 collapse, 2 cluster
 // pairs), scheme, storage and tiling: the attribute set by it stays with the function.
-cudaError_t prepared(int kind, int Q, int prec, int S, int NT, int* out) {
+cudaError_t prepared(int kind, int Q, int prec, int S, int NT, bool zb, int* out) {
   static std::mutex mu;
-  static std::map<std::array<int, 6>, int> done;
+  static std::map<std::array<int, 7>, int> done;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  const std::array<int, 6> key{dev, kind, Q, prec, S, NT};
+  const std::array<int, 7> key{dev, kind, Q, prec, S, NT, zb ? 1 : 0};
   std::lock_guard<std::mutex> lock(mu);
   auto it = done.find(key);
   if (it == done.end()) {
     int v = 0;
-    e = kind == 0 ? resident_prepare(Q, prec, S, NT, &v)
-        : kind == 1 ? collapse_resident_prepare(Q, prec, S, NT, &v)
-                    : resident_cluster_prepare(Q, prec, S, NT, &v);
+    e = kind == 0 ? resident_prepare(Q, prec, S, NT, zb, &v)
+        : kind == 1 ? collapse_resident_prepare(Q, prec, S, NT, zb, &v)
+                    : resident_cluster_prepare(Q, prec, S, NT, zb, &v);
     if (e != cudaSuccess) return e;  // not kept: the caller clears the error and tries another tiling
     it = done.emplace(key, v).first;
   }
@@ -467,10 +468,10 @@ int setup_resident(lb_ks* h, bool required, int S_force = 0, int NT_force = 0, d
     for (const Piece& p : rings) nhalves += p.halo > 0 ? 1 : 0;
     pack_blocks(segs, NT, &segbins);
     int bps = 0, max_clusters = 0;
-    cudaError_t e = prepared(col ? 1 : 0, h->Q, h->prec, S, NT, &bps);
+    cudaError_t e = prepared(col ? 1 : 0, h->Q, h->prec, S, NT, h->zb, &bps);
     if (e != cudaSuccess || bps < 1) { cudaGetLastError(); continue; }
     if (!pairs.used.empty()) {
-      e = prepared(2, h->Q, h->prec, S, NT, &max_clusters);
+      e = prepared(2, h->Q, h->prec, S, NT, h->zb, &max_clusters);
       if (e != cudaSuccess || max_clusters < 1) { cudaGetLastError(); continue; }
     }
     const int slots = bps * sms;  // resident blocks
@@ -530,7 +531,7 @@ int issue_lane(lb_ks* h, const Lane& L, int64_t k, int from, bool in_place, cuda
     if (!h->blocked) LBKS_CUDA(h, cudaMemsetAsync(L.d_queue, 0, sizeof(int), s), "queue reset");
     ResidentLaunch RL{h->Q, h->prec, h->S, h->NT, arena(h, cur), arena(h, dst), h->d_runs,
                       L.d_pieces, L.d_bundles, L.nbundles, L.d_queue, (int)kk, L.grid, L.cl, h->d_flags,
-                      h->nplanes == 1, L.kx, h->link_wait_limit, h->link_withhold_step, L.one, L.spread};
+                      h->nplanes == 1, L.kx, h->link_wait_limit, h->link_withhold_step, L.one, L.spread, h->zb};
     LBKS_CUDA(h, h->blocked ? launch_blocked(RL, h->reservoir, s) : launch_resident(RL, s), "resident step");
     *nk += 1;
     cur = dst;
@@ -773,6 +774,19 @@ int autotune_resident(lb_ks* h) {
   return LB_KS_OK;
 }
 
+// Whether the operations that the Z instances of the kernels leave out add zero in every
+// run: the c = +-3 planes' rho^2 terms (D1Q7's first-moment weights are zero there, except
+// with the full-inverse ablation), and for the FP64 collapse rhobar.
+bool zero_terms(const lb_ks* h) {
+  const bool col64 = h->nplanes == 1 && h->prec == kF64;
+  if (h->Q != 7 && h->nplanes != 1) return false;
+  for (const RunDesc& d : h->runs_h) {
+    if (h->Q == 7 && (d.b[5] != 0.0 || d.b[6] != 0.0 || d.B[5] != 0.0 || d.B[6] != 0.0)) return false;
+    if (col64 && d.rhobar != 0.0) return false;
+  }
+  return true;
+}
+
 int check_flags(lb_ks* h) {
   int flag = 0;
   LBKS_CUDA(h, cudaMemcpy(&flag, h->d_flags, sizeof(int), cudaMemcpyDeviceToHost), "read flags");
@@ -960,6 +974,7 @@ int create_body(lb_ks*& h, lb_ks_t** out, int scheme, int32_t nruns, const int64
     off += align_up(N[r] + 2 * ghost, kAlign);
   }
   h->plane = std::max<int64_t>(off, kAlign);
+  h->zb = zero_terms(h);  // (rhobar is still zero here, as it stays in FP64)
 
   // Tiles.  The streaming tiles (also those of the guard, the statistics of rho0 and the
   // gathers) always; the plain family's only when a kernel that uses them runs (the
@@ -1360,6 +1375,16 @@ int lb_ks_load(lb_ks_t* h, const void* buf, size_t bytes) try {
   h->mass0_h = m0;
   h->tables_on_host = true;
   LBKS_CUDA(h, cudaMemcpy(h->d_runs, runs.data(), sizeof(RunDesc) * h->nruns, cudaMemcpyHostToDevice), "load runs");
+  if (h->zb && !zero_terms(h)) {
+    // the loaded constants have such a term: the general kernels from now on
+    h->zb = false;
+    for (auto& g : h->graphs) cudaGraphExecDestroy(g.exec);
+    h->graphs.clear();
+    int v = 0;
+    for (int l = 0; l < h->nlanes && !h->blocked; ++l)
+      LBKS_CUDA(h, prepared(h->nplanes == 1 ? 1 : (h->lanes[l].cl == 2 ? 2 : 0), h->Q, h->prec, h->S, h->NT, false, &v),
+                "prepare kernels");
+  }
   if (h->prec == kF64) LBKS_CUDA(h, launch_fix_coef(h->Q, h->nruns, h->d_runs, h->stream), "load runs");
   LBKS_CUDA(h, cudaMemcpy(h->d_mass0, m0.data(), sizeof(double) * h->nruns, cudaMemcpyHostToDevice), "load mass0");
   LBKS_CUDA(h, cudaMemcpy(h->fbuf[h->cur], p, storage_bytes(h->prec) * (size_t)h->nplanes * (size_t)h->plane,

@@ -45,17 +45,20 @@ __device__ __forceinline__ CollapseCoef<CT, C> load_collapse_coef(const RunDesc&
 // of 2 c_max, which in FP32 would bias the slow long-wave modes.  Every kernel of
 // the collapse family calls this with the same operands, so their results agree
 // bitwise.
-template <typename CT, int C>
+// ZB: B_3 is zero (D1Q7's default weights), so that its term, four of the 22 operations, is
+// an addition of zero.  ZR: rhobar is zero (FP64 storage), and so is what is added to s.
+template <typename CT, int C, bool ZB = false, bool ZR = false>
 __device__ __forceinline__ CT collapse_site(CT d0, const CT (&dl)[C + 1], const CT (&dr)[C + 1],
                                             const CollapseCoef<CT, C>& k) {
   CT inc = CT(0);
 #pragma unroll
   for (int c = 1; c <= C; ++c) {
     const CT s = add_rn(dl[c], dr[c]);
-    const CT df = add_rn(dl[c], -dr[c]);
     const CT lap = fma_rn(CT(-2), d0, s);                  // rho(x-c) + rho(x+c) - 2 rho(x)
-    const CT q = mul_rn(df, add_rn(k.two_rhobar, s));      // rho(x-c)^2 - rho(x+c)^2
     inc = fma_rn(k.A[c], lap, inc);
+    if (ZB && c == 3) continue;
+    const CT df = add_rn(dl[c], -dr[c]);
+    const CT q = mul_rn(df, ZR ? s : add_rn(k.two_rhobar, s));  // rho(x-c)^2 - rho(x+c)^2
     inc = fma_rn(k.B[c], q, inc);
   }
   return add_rn(d0, inc);

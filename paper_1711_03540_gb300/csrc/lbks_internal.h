@@ -130,10 +130,11 @@ struct ResidentLaunch {
   int withhold_step = -1;          // cl = 2, testing aid: block 1 sends nothing across the edge at this step
   bool one = false;                // blocked kernel: every bundle holds one piece
   bool spread = false;             // ... and there is at most one block per SM
+  bool zb = false;                 // D1Q7: b is zero for c = +-3 in every run; FP64 collapse: rhobar too
 };
 bool resident_supported(int Q, int storage, int S, int NT);
 size_t resident_smem(int Q, int storage, int S, int NT);  // dynamic shared memory of a block
-cudaError_t resident_prepare(int Q, int storage, int S, int NT, int* blocks_per_sm);
+cudaError_t resident_prepare(int Q, int storage, int S, int NT, bool zb, int* blocks_per_sm);
 // The tau = 1 collapse (one stored plane).
 int collapse_tile_sites();
 cudaError_t launch_collapse_init(int storage, Arena dst, const RunDesc* runs, const Tile* tiles, int ntiles,
@@ -141,11 +142,11 @@ cudaError_t launch_collapse_init(int storage, Arena dst, const RunDesc* runs, co
 cudaError_t launch_collapse_step(int Q, int storage, Arena src, Arena dst, const RunDesc* runs, const Tile* tiles,
                                  int ntiles, cudaStream_t s);
 bool collapse_resident_supported(int Q, int storage, int S, int NT);
-cudaError_t collapse_resident_prepare(int Q, int storage, int S, int NT, int* blocks_per_sm);
+cudaError_t collapse_resident_prepare(int Q, int storage, int S, int NT, bool zb, int* blocks_per_sm);
 cudaError_t launch_collapse_resident(const ResidentLaunch& L, cudaStream_t s);
 
 // Clusters of two blocks: the largest number of clusters resident at once.
-cudaError_t resident_cluster_prepare(int Q, int storage, int S, int NT, int* max_clusters);
+cudaError_t resident_cluster_prepare(int Q, int storage, int S, int NT, bool zb, int* max_clusters);
 cudaError_t launch_resident_cluster(const ResidentLaunch& L, cudaStream_t s);
 cudaError_t launch_resident(const ResidentLaunch& L, cudaStream_t s);
 

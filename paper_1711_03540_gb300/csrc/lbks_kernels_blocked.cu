@@ -142,12 +142,13 @@ __global__ void __launch_bounds__(NTM, MINB)
 // The tau = 1 collapse in the same form: one value per thread, its 2 c_max neighbours read
 // from the exchange area each step (with the guard columns for wrapping ends).  FP64
 // storage, FP32 batches too small for the register-resident collapse, and reservoir ends
-// (the fixed nodes keep their values, put in both parities once).  FP64 is bound by the
+// (the fixed nodes keep their values, put in both parities once).  Z: the operations that
+// add zero are left out (collapse_site's ZB, and ZR in FP64).  FP64 is bound by the
 // FP64 pipe, so what counts is to use every SM's: one 4096-site lattice 25 -> 1.0 us per
 // step, 24 lattices 25 -> 3.9, the 4096-lattice ensemble 442 -> 418; FP32, 24 lattices: 1.02
 // -> 0.34 us, one lattice 0.57 -> 0.20 (300 lattices: 1.03 either way, so larger batches
 // stay register-resident).
-template <int C, int ST, bool RES, bool ONE>
+template <int C, int ST, bool RES, bool ONE, bool Z>
 __global__ void __launch_bounds__(512, 2)
     blocked_collapse_kernel(Arena src, Arena dst, const RunDesc* __restrict__ runs, const Piece* __restrict__ pieces,
                             const int2* __restrict__ bundles, int ksteps) {
@@ -195,7 +196,7 @@ __global__ void __launch_bounds__(512, 2)
         dl[c] = xs[-c];
         dr[c] = xs[c];
       }
-      v = collapse_site<CT, C>(v, dl, dr, k);
+      v = collapse_site<CT, C, Z, Z && ST == kF64>(v, dl, dr, k);
     }
   }
   if (active && !fixed && j >= pc.st_lo && j < pc.st_hi) static_cast<T*>(dst.f)[d.off + x] = static_cast<T>(v);
@@ -227,14 +228,19 @@ cudaError_t launch_t(const ResidentLaunch& L, cudaStream_t s) {
   }
 }
 
-template <int Q, int ST, bool RES>
-cudaError_t launch_collapse_t(const ResidentLaunch& L, cudaStream_t s) {
+template <int Q, int ST, bool RES, bool Z>
+cudaError_t launch_collapse_z(const ResidentLaunch& L, cudaStream_t s) {
   constexpr int C = cmax_of(Q);
   if (L.one)
-    return launch_early(blocked_collapse_kernel<C, ST, RES, true>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs, L.pieces,
-                        L.bundles, L.ksteps);
-  return launch_early(blocked_collapse_kernel<C, ST, RES, false>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs, L.pieces,
-                      L.bundles, L.ksteps);
+    return launch_early(blocked_collapse_kernel<C, ST, RES, true, Z>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs,
+                        L.pieces, L.bundles, L.ksteps);
+  return launch_early(blocked_collapse_kernel<C, ST, RES, false, Z>, L.nbundles, L.NT, 0, s, L.src, L.dst, L.runs,
+                      L.pieces, L.bundles, L.ksteps);
+}
+
+template <int Q, int ST, bool RES>
+cudaError_t launch_collapse_t(const ResidentLaunch& L, cudaStream_t s) {
+  return L.zb ? launch_collapse_z<Q, ST, RES, true>(L, s) : launch_collapse_z<Q, ST, RES, false>(L, s);
 }
 
 #define LBKS_BLOCKED_DISPATCH(OP)                                                    \

@@ -139,7 +139,7 @@ struct CollapseResidentArgs {
   int ksteps;
 };
 
-template <int C, int ST, int S>
+template <int C, int ST, int S, bool ZB>
 __global__ void __launch_bounds__(kCRThreads, 1) collapse_resident_kernel(const CollapseResidentArgs a) {
   using T = typename StorageType<ST>::type;
   using CT = typename StorageType<ST>::compute;
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kCRThreads, 1) collapse_resident_kernel(const 
             dl[c] = e[C + s - c];
             dr[c] = e[C + s + c];
           }
-          nw[s] = collapse_site<CT, C>(e[C + s], dl, dr, k);
+          nw[s] = collapse_site<CT, C, ZB>(e[C + s], dl, dr, k);
         }
 #pragma unroll
         for (int s = 0; s < S; ++s) e[C + s] = nw[s];
@@ -300,21 +300,21 @@ size_t cr_smem_bytes(int NT) {
     default: break;                                    \
   }
 
-template <int C, int ST, int S>
+template <int C, int ST, int S, bool ZB>
 cudaError_t cr_prepare_t(int NT, int* blocks_per_sm) {
   // the opt-in covers the largest block (kCRThreads), so that preparing a smaller tiling
   // later never lowers it under a larger one already prepared
   const size_t smem = cr_smem_bytes<C, ST, S>(NT);
-  cudaError_t e = cudaFuncSetAttribute(collapse_resident_kernel<C, ST, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(collapse_resident_kernel<C, ST, S, ZB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)cr_smem_bytes<C, ST, S>(kCRThreads));
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, collapse_resident_kernel<C, ST, S>, NT, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, collapse_resident_kernel<C, ST, S, ZB>, NT, smem);
 }
 
-template <int C, int ST, int S>
+template <int C, int ST, int S, bool ZB>
 cudaError_t cr_launch_t(const ResidentLaunch& L, cudaStream_t s) {
   const CollapseResidentArgs a{L.src, L.dst, L.runs, L.pieces, L.bundles, L.nbundles, L.queue, L.ksteps};
-  collapse_resident_kernel<C, ST, S><<<L.grid, L.NT, cr_smem_bytes<C, ST, S>(L.NT), s>>>(a);
+  collapse_resident_kernel<C, ST, S, ZB><<<L.grid, L.NT, cr_smem_bytes<C, ST, S>(L.NT), s>>>(a);
   return cudaGetLastError();
 }
 
@@ -328,9 +328,10 @@ bool collapse_resident_supported(int Q, int storage, int S, int NT) {
   return NT >= 32 && NT <= kCRThreads && NT % 32 == 0;
 }
 
-cudaError_t collapse_resident_prepare(int Q, int storage, int S, int NT, int* blocks_per_sm) {
+cudaError_t collapse_resident_prepare(int Q, int storage, int S, int NT, bool zb, int* blocks_per_sm) {
   if (!collapse_resident_supported(Q, storage, S, NT)) return cudaErrorInvalidValue;
-  LBKS_COLLAPSE_CASES(return (cr_prepare_t<Cc, STc, Sc>(NT, blocks_per_sm)));
+  LBKS_COLLAPSE_CASES(if (Cc == 3 && zb) return (cr_prepare_t<Cc, STc, Sc, Cc == 3>(NT, blocks_per_sm));
+                      return (cr_prepare_t<Cc, STc, Sc, false>(NT, blocks_per_sm)));
   return cudaErrorInvalidValue;
 }
 
@@ -338,7 +339,8 @@ cudaError_t launch_collapse_resident(const ResidentLaunch& L, cudaStream_t s) {
   const int Q = L.Q, storage = L.storage, S = L.S;
   if (!collapse_resident_supported(Q, storage, S, L.NT) || L.cl != 1) return cudaErrorInvalidValue;
   if (L.nbundles == 0 || L.grid == 0) return cudaSuccess;
-  LBKS_COLLAPSE_CASES(return (cr_launch_t<Cc, STc, Sc>(L, s)));
+  LBKS_COLLAPSE_CASES(if (Cc == 3 && L.zb) return (cr_launch_t<Cc, STc, Sc, Cc == 3>(L, s));
+                      return (cr_launch_t<Cc, STc, Sc, false>(L, s)));
   return cudaErrorInvalidValue;
 }
 

@@ -377,18 +377,20 @@ inline std::vector<int> by_threads_desc(const std::vector<Piece>& pieces) {
 // Time of a step of the register-resident kernel (D1Q7, microseconds), S sites per thread
 // and q warps on each of an SM's schedulers, measured on single lattices and on uniform
 // batches that fill the device; 0: not a tiling that choose_resident considers.  Two blocks
-// of 128 threads overlap one's barrier with the other's step: 14 to 17 % less per site than
-// one of 256 (1.07e12 and 1.08e12 site-updates/s at 18 and 16 sites, 0.92e12 at 20 x 256).
-inline double resident_step_us(int S, int NT, int q) {
-  if (NT == 128 && q == 2 && (S == 18 || S == 16)) return S == 18 ? 0.654 : 0.575;
+// of 128 threads overlap one's barrier with the other's step (1.11e12 and 1.13e12
+// site-updates/s at 18 and 16 sites, 1.10e12 at 16 x 256, 0.94e12 at 20 x 256).  pairs: the
+// cluster kernel, whose 16-site loop is scheduled worse, with the halves' exchanges.
+inline double resident_step_us(int S, int NT, int q, bool pairs) {
+  if (pairs && q == 2) return (NT < 256 ? 1.2 : 1.0) * (S == 20 ? 0.866 : S == 18 ? 0.80 : S == 16 ? 0.756 : 0.9);
+  if (NT == 128 && q == 2 && (S == 18 || S == 16)) return S == 18 ? 0.629 : 0.549;
   const auto at = [q](double first, double more) { return first + more * (q - 1); };
   switch (S) {
-    case 20: return at(0.48, 0.375);
-    case 18: return at(0.385, 0.335);
-    case 16: return at(0.345, 0.315);
-    case 8: return at(0.285, 0.175);
-    case 6: return at(0.26, 0.127);
-    case 4: return at(0.235, 0.10);
+    case 20: return at(0.48, 0.35);
+    case 18: return at(0.385, 0.32);
+    case 16: return at(0.345, 0.225);
+    case 8: return at(0.285, 0.145);
+    case 6: return at(0.26, 0.105);
+    case 4: return at(0.235, 0.09);
     default: return 0.0;
   }
 }
@@ -411,7 +413,7 @@ struct ResidentTiling {
 // sites; kseg is the cheapest, or kfix.
 inline ResidentTiling rate_resident(const std::vector<int64_t>& Ns, int Q, int S, int NT, int bps, int sms, bool f16,
                                     int kmax, bool may_spread, int kfix = 0) {
-  const double edge = S == 18 ? 14.5 : 20.0, half_cost = NT < 256 ? 1.2 : 1.05;
+  const double edge = S == 18 ? 14.5 : 20.0;
   constexpr double kLaunchUs = 3.0, kRingCost = 1.4, kRingUs = 0.4;
   const int C = (Q - 1) / 2, h = C * kPairStepsMax;
   const double scale = Q == 7 ? 1.0 : 0.7;
@@ -448,25 +450,24 @@ inline ResidentTiling rate_resident(const std::vector<int64_t>& Ns, int Q, int S
     if (b == room.size()) room.push_back(NT);
     room[b] -= v;
   }
-  const double blocks = ((double)room.size() * (1.0 + (half_cost - 1.0) * (double)halves / std::max<double>(1.0, (double)threads.size())) +
-                         2.0 * kRingCost * (double)rings) * (double)stride;
+  const double blocks = ((double)room.size() + 2.0 * kRingCost * (double)rings) * (double)stride;
   const double slots = (double)sms * bps;
-  const auto warps = [&](double per_sm, int64_t threads) {  // per scheduler
-    return (int)std::ceil(per_sm * (double)((threads + 31) / 32) / 4.0 - 1e-9);
+  const auto warps = [&](double per_sm, int64_t threads) {  // per scheduler: a block's first warp is the first's
+    return (int)std::ceil(per_sm - 1e-9) * (int)((threads + 127) / 128);
   };
   double us = rings ? kRingUs : 0.0;
   if (pieces > 0.0) {
     t.spread = may_spread && !pairs && cut.empty() && pieces <= slots;
     if (t.spread) {
-      us = scale * resident_step_us(S, NT, warps(std::ceil(pieces / sms), widest));
+      us = scale * resident_step_us(S, NT, warps(std::ceil(pieces / sms), widest), false);
     } else {
       const double rounds = std::ceil(blocks / slots);
-      us = scale * rounds * resident_step_us(S, NT, warps(std::min<double>(bps, std::ceil(blocks / sms)), NT));
+      us = scale * rounds * resident_step_us(S, NT, warps(std::min<double>(bps, std::ceil(blocks / sms)), NT), pairs);
     }
   }
   if (!cut.empty()) {
     if (f16) return t;
-    const double full = scale * resident_step_us(S, NT, warps(bps, NT));
+    const double full = scale * resident_step_us(S, NT, warps(bps, NT), false);
     double best = 1e300;
     for (int k = kfix ? kfix : 16; k <= std::min(kmax, 192); k += 8) {
       const int64_t room = (int64_t)NT * S - 2LL * C * k - 2 * S;

@@ -214,13 +214,23 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* m, uint32_t parity) {
   return ok != 0;
 }
 
+// Post-collision value of one plane (post_collision in lbks_device.cuh).  NOB: the plane's
+// b is zero, so that rho^2 b + t is t: the c = +-3 planes of D1Q7, whose first-moment
+// weights w1 are zero (Sec. 2.3; not with the full-inverse weights), saving 2 of a site's 29
+// FP32 instructions.
+template <bool NOB, typename CT>
+__device__ __forceinline__ CT post_plane(CT r, CT g, CT rho2, CT b, CT t) {
+  if constexpr (NOB) return fma_rn(r, g, t);
+  else return fma_rn(r, g, fma_rn(rho2, b, t));
+}
+
 // Edge values of one thread for the other block of a cluster: the post-collision
 // values of its last k + 1 slots for each speed +k (push_edge_right) or of its first
 // k + 1 for each -k (push_edge_left), from the pre-collision populations f and phase
 // A's rho and rho^2, with the operations of phase B (which computes the same values
 // again below), stored into the other block's pushed-in column (cluster address col,
 // element stride ntx, the rows of phase B's own column).
-template <int Q, typename CT, int S>
+template <int Q, bool ZB, typename CT, int S>
 __device__ __forceinline__ void push_edge_right(const CT (&f)[Q][S], const CT (&rho)[S], const CT (&rho2)[S],
                                                 const Coef<CT, Q>& k, uint32_t col, int ntx) {
   StaticFor<1, Q>::run([&](auto ic) {
@@ -230,14 +240,14 @@ __device__ __forceinline__ void push_edge_right(const CT (&f)[Q][S], const CT (&
 #pragma unroll
       for (int j = 0; j <= c; ++j) {
         constexpr int s0 = S - 1 - c;
-        const CT v = post_collision(k.r, f[i][s0 + j], rho[s0 + j], rho2[s0 + j], k.b[i], mul_rn(rho[s0 + j], k.a[i]));
+        const CT v = post_plane<ZB && c == 3>(k.r, f[i][s0 + j], rho2[s0 + j], k.b[i], mul_rn(rho[s0 + j], k.a[i]));
         st_cluster(col + (uint32_t)((xrow(c) + j) * ntx * sizeof(CT)), v);
       }
     }
   });
 }
 
-template <int Q, typename CT, int S>
+template <int Q, bool ZB, typename CT, int S>
 __device__ __forceinline__ void push_edge_left(const CT (&f)[Q][S], const CT (&rho)[S], const CT (&rho2)[S],
                                                const Coef<CT, Q>& k, uint32_t col, int ntx) {
   StaticFor<1, Q>::run([&](auto ic) {
@@ -249,7 +259,7 @@ __device__ __forceinline__ void push_edge_left(const CT (&f)[Q][S], const CT (&r
       for (int j = 0; j <= kk; ++j) {
         // phase B takes rho a_i of the -c plane from the +c plane before it (a_i is even in
         // c) and b_i as minus that plane's (b_i is odd in c, exactly)
-        const CT v = post_collision(k.r, f[i][j], rho[j], rho2[j], -k.b[i - 1], mul_rn(rho[j], k.a[i - 1]));
+        const CT v = post_plane<ZB && kk == 3>(k.r, f[i][j], rho2[j], -k.b[i - 1], mul_rn(rho[j], k.a[i - 1]));
         st_cluster(col + (uint32_t)((xrow(kk) + j) * ntx * sizeof(CT)), v);
       }
     }
@@ -299,7 +309,7 @@ struct ClusterLink {
 // barrier is the named barrier 1 over the nbar threads of the warps that hold one; with
 // LINK every thread steps (those without a piece on zeros), so that every thread keeps
 // the link's phase parities.
-template <int Q, int S, int XS, bool LINK, bool SKIP, typename CT>
+template <int Q, int S, int XS, bool LINK, bool SKIP, bool ZB, typename CT>
 __device__ __forceinline__ void resident_steps(CT (&f)[Q][S], const Coef<CT, Q>& k, const int step0, const int ksteps,
                                                CT* const xbase, const int t, const bool active, const bool full,
                                                const int lt, const int rt, const bool lfull, const bool wrun,
@@ -385,12 +395,12 @@ __device__ __forceinline__ void resident_steps(CT (&f)[Q][S], const Coef<CT, Q>&
           // receiver: 7 % slower rings.
           if (step != ln.withhold) {
             if (ln.rrem) {
-              push_edge_right<Q>(f, rho, rho2, k, ln.peer_x + (uint32_t)((pb * 2 * NR * NTX + XS - 2) * sizeof(CT)),
+              push_edge_right<Q, ZB>(f, rho, rho2, k, ln.peer_x + (uint32_t)((pb * 2 * NR * NTX + XS - 2) * sizeof(CT)),
                                  NTX);
               mbar_arrive_remote(ln.peer_mbar + 8u * pb);
             }
             if (ln.lrem) {
-              push_edge_left<Q>(f, rho, rho2, k,
+              push_edge_left<Q, ZB>(f, rho, rho2, k,
                                 ln.peer_x + (uint32_t)(((pb * 2 + 1) * NR * NTX + XS - 1) * sizeof(CT)), NTX);
               mbar_arrive_remote(ln.peer_mbar + 8u * pb);
             }
@@ -407,7 +417,7 @@ __device__ __forceinline__ void resident_steps(CT (&f)[Q][S], const Coef<CT, Q>&
 #pragma unroll
             for (int s = S - 1; s >= 0; --s) {
               tt[s] = mul_rn(rho[s], k.a[i]);  // shared with the -c plane that follows
-              const CT v = post_collision(k.r, f[i][s], rho[s], rho2[s], k.b[i], tt[s]);
+              const CT v = post_plane<ZB && kk == 3>(k.r, f[i][s], rho2[s], k.b[i], tt[s]);
               f[0][s] = add_rn(f[0][s], -v);
               if (s >= S - 1 - kk) xw[(row0 + s - (S - 1 - kk)) * NTX] = v;
               if (s + kk <= S - 1) f[i][s + kk] = v;
@@ -417,7 +427,7 @@ __device__ __forceinline__ void resident_steps(CT (&f)[Q][S], const Coef<CT, Q>&
             for (int s = 0; s < S; ++s) {
               // b_i of the -c plane is exactly minus the +c plane's (B_i = J w1_i, w1 odd in
               // c), taken with the FMA's negation so that it needs no register of its own
-              const CT v = post_collision(k.r, f[i][s], rho[s], rho2[s], -k.b[i - 1], tt[s]);
+              const CT v = post_plane<ZB && kk == 3>(k.r, f[i][s], rho2[s], -k.b[i - 1], tt[s]);
               f[0][s] = add_rn(f[0][s], -v);
               if (s <= kk) xw[(NR + row0 + s) * NTX] = v;
               if (s >= kk) f[i][s - kk] = v;
@@ -564,7 +574,8 @@ __device__ __forceinline__ PieceGeom piece_geom(const Piece& pc, const int64_t N
   return G;
 }
 
-template <int Q, int ST, int S, int CL>
+// ZB: b is zero for the c = +-3 planes of every run (post_plane).
+template <int Q, int ST, int S, int CL, bool ZB>
 __global__ void __launch_bounds__(ResidentCfg<ST, S>::kMaxThreads, 1) resident_kernel(const ResidentArgs a) {
   static_assert(CL == 1 || CL == 2, "work groups are one block or a pair of blocks");
   using T = typename StorageType<ST>::type;
@@ -711,7 +722,7 @@ __global__ void __launch_bounds__(ResidentCfg<ST, S>::kMaxThreads, 1) resident_k
         ln.flags = a.flags;
         ln.limit = a.wait_limit;
         ln.withhold = rank == 1 ? a.withhold_step : -1;
-        resident_steps<Q, S, NTX, true, kSkip>(f, k, 0, a.ksteps, xbase, t, active, full, lt, rt, lfull, wrun, nbar, ln);
+        resident_steps<Q, S, NTX, true, kSkip, ZB>(f, k, 0, a.ksteps, xbase, t, active, full, lt, rt, lfull, wrun, nbar, ln);
         // every thread toggled the same parities; the next write follows the barriers
         // of the store phase below
         if (t == 0) s_ph = ln.ph;
@@ -719,15 +730,15 @@ __global__ void __launch_bounds__(ResidentCfg<ST, S>::kMaxThreads, 1) resident_k
       } else if (halves && a.kx > 0) {
         for (int s0 = 0; s0 < a.ksteps; s0 += a.kx) {
           const int kk = min(a.kx, a.ksteps - s0);
-          resident_steps<Q, S, NTX, false, kSkip>(f, k, s0, kk, xbase, t, active, full, lt, rt, lfull, wrun, nbar, ln);
+          resident_steps<Q, S, NTX, false, kSkip, ZB>(f, k, s0, kk, xbase, t, active, full, lt, rt, lfull, wrun, nbar, ln);
           if (s0 + kk < a.ksteps)
             halo_exchange<Q, S>(f, s_half, full, start, NT, t, stage, inbox, (s0 / a.kx) & 1);
         }
       } else {
-        resident_steps<Q, S, NTX, false, kSkip>(f, k, 0, a.ksteps, xbase, t, active, full, lt, rt, lfull, wrun, nbar, ln);
+        resident_steps<Q, S, NTX, false, kSkip, ZB>(f, k, 0, a.ksteps, xbase, t, active, full, lt, rt, lfull, wrun, nbar, ln);
       }
     } else {
-      resident_steps<Q, S, NTX, false, kSkip>(f, k, 0, a.ksteps, xbase, t, active, full, lt, rt, lfull, wrun, nbar, ln);
+      resident_steps<Q, S, NTX, false, kSkip, ZB>(f, k, 0, a.ksteps, xbase, t, active, full, lt, rt, lfull, wrun, nbar, ln);
     }
     __syncthreads();
 
@@ -767,6 +778,9 @@ size_t smem_bytes_t(int NT) {
   using CT = typename StorageType<ST>::compute;
   return sizeof(CT) * smem_elems(Q, S, NT, ResidentCfg<ST, S>::kXS);
 }
+
+// Which instance runs a launch: ZB is compiled for D1Q7 in FP32 arithmetic alone.
+template <int Q, int ST> constexpr bool has_zb() { return Q == 7 && ST != kF64; }
 
 #define LBKS_RESIDENT_CASES(Q_, ST_, OP)                                              \
   if (Q == Q_ && storage == ST_) {                                                    \
