@@ -459,7 +459,8 @@ def resident_fp64(lb, torch, wl, stream, local, steps=3, warmup=1):
         lb.lb_ks_free(h)
     v = wl.sites * LB_STEPS_PER_STEP * steps / (tot * 1e-3)
     tf = v * FLOP_PER_SITE_UPDATE[wl.scheme] / 1e12
-    return {"value": v, "unit": "site-updates/s", "kernel": "resident_kernel<7,F64,%d>" % desc["sites_per_thread"],
+    return {"value": v, "unit": "site-updates/s", "kernel": ("blocked_step_kernel<7,F64>" if desc["sites_per_thread"] == 1 else
+                       "resident_kernel<7,F64,%d>" % desc["sites_per_thread"]),
             "threads_per_block": desc["threads_per_block"], "steps_timed": steps * LB_STEPS_PER_STEP,
             "tflops": tf, "frac_of_nominal_fp64": tf / FP64_NOMINAL_TFLOPS, "gpu_launches": int(nl), "clocks": clocks}
 

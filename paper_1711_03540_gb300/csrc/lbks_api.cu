@@ -349,22 +349,23 @@ int setup_blocked(lb_ks* h, int sms, double than) {
   if (b.NT == 0 || b.us >= than) return 1;
   std::vector<Piece> pieces;
   if (!plan_blocked(h->N, h->reservoir, h->cmax, b.NT, b.k, &pieces)) return 1;
-  std::vector<Piece> ordered;
-  std::vector<int2> bundles;
-  blocked_bundles(pieces, b.NT, b.spread, &ordered, &bundles);
   bool segmented = false;
   for (const Piece& p : pieces) segmented = segmented || p.st_hi - p.st_lo < p.n;
+  std::vector<int2> bundles;
+  blocked_bundles(pieces, b.NT, b.spread, &bundles);
   Lane& L = h->lanes[0];
   int rc;
-  if ((rc = upload_lane(h, &L, ordered, bundles, 1, b.k, segmented, 1.0))) return rc;
+  if ((rc = upload_lane(h, &L, pieces, bundles, 1, b.k, segmented, 1.0))) return rc;
+  if (bundles.empty()) L.nbundles = (int)pieces.size();
   L.grid = L.nbundles;
-  L.one = bundles.size() == pieces.size();
+  L.one = bundles.empty();
   L.spread = b.spread && L.nbundles <= sms;
   h->nlanes = 1;
   h->blocked = true;
   h->S = 1;
   h->NT = b.NT;
-  h->kmax = h->kseg = b.k;
+  h->kmax = b.k;
+  h->kseg = segmented ? b.k : 1;
   return LB_KS_OK;
 }
 
@@ -703,7 +704,7 @@ int autotune_resident(lb_ks* h) {
   std::vector<Cand> cands;
   std::vector<std::pair<int, int>> tilings;
   const bool col = h->nplanes == 1;  // the tau = 1 collapse's resident kernel
-  if (free_tiling(h)) cands.push_back({0, 0, 1.25, 0, -1, -1});  // the choice by size
+  if (free_tiling(h)) cands.push_back({0, 0, 1.0, 0, -1, -1});  // the choice by size
   if (h->opts.sites_per_thread) {
     tilings.push_back({h->opts.sites_per_thread, h->opts.threads_per_block});
   } else if (col) {

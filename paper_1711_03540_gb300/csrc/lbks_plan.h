@@ -574,28 +574,25 @@ inline void pack_blocks(std::vector<Piece>& pieces, int NT, Bins* blocks) {
 
 // Bundles of the one-site-per-thread kernel: each stretch of a longer lattice has a block of
 // its own (stretches of a lattice are equally long and fill most of it); whole lattices
-// too when spread, else packed first fit after them.
-inline void blocked_bundles(const std::vector<Piece>& pieces, int NT, bool spread, std::vector<Piece>* ordered,
-                            std::vector<int2>* bundles) {
-  ordered->clear();
+// too when spread, else packed first fit after them.  `pieces` is put in bundle order;
+// `bundles` is left empty when every piece is a bundle of its own.
+inline void blocked_bundles(std::vector<Piece>& pieces, int NT, bool spread, std::vector<int2>* bundles) {
   bundles->clear();
-  ordered->reserve(pieces.size());
-  std::vector<Piece> whole;
+  const auto whole = [](const Piece& p) { return p.st_lo == 0 && p.st_hi == p.n; };
+  if (spread || std::none_of(pieces.begin(), pieces.end(), whole)) return;
+  std::vector<Piece> small, packed;
+  std::vector<int2> more;
+  size_t n = 0;
   for (const Piece& p : pieces) {
-    if (!spread && p.st_lo == 0 && p.st_hi == p.n) {
-      whole.push_back(p);
-    } else {
-      bundles->push_back(int2{(int)ordered->size(), 1});
-      ordered->push_back(p);
-    }
+    if (whole(p)) small.push_back(p);
+    else pieces[n++] = p;
   }
   Bins bins;
-  pack_blocks(whole, NT, &bins);
-  std::vector<Piece> packed;
-  std::vector<int2> more;
-  bins.emit(whole, &packed, &more);
-  for (int2 b : more) bundles->push_back(int2{b.x + (int)ordered->size(), b.y});
-  ordered->insert(ordered->end(), packed.begin(), packed.end());
+  pack_blocks(small, NT, &bins);
+  bins.emit(small, &packed, &more);
+  for (size_t b = 0; b < n; ++b) bundles->push_back(int2{(int)b, 1});
+  for (int2 b : more) bundles->push_back(int2{b.x + (int)n, b.y});
+  std::copy(packed.begin(), packed.end(), pieces.begin() + (int64_t)n);
 }
 
 }  // namespace plan

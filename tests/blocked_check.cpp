@@ -10,11 +10,14 @@ using namespace lbks::plan;
 
 // 0 if the plan holds every site once with its halo and no two pieces share a thread.
 static int check(const std::vector<int64_t>& Ns, bool res, int C, int NT, int k, bool spread) {
-  std::vector<Piece> pieces, ordered;
+  std::vector<Piece> pieces;
   std::vector<int2> bundles;
   if (!plan_blocked(Ns, res, C, NT, k, &pieces)) return NT - 2 * C * k > 0 ? 1 : 0;
-  blocked_bundles(pieces, NT, spread, &ordered, &bundles);
+  std::vector<Piece> ordered = pieces;
+  blocked_bundles(ordered, NT, spread, &bundles);
   if (ordered.size() != pieces.size()) return 2;
+  if (bundles.empty())  // one piece each
+    for (size_t b = 0; b < ordered.size(); ++b) bundles.push_back(int2{(int)b, 1});
   std::vector<std::vector<int>> seen(Ns.size());
   const int ghost = res ? C : 0;
   for (size_t r = 0; r < Ns.size(); ++r) seen[r].assign((size_t)(Ns[r] + 2 * ghost), 0);
