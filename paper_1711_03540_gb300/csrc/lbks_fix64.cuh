@@ -23,8 +23,8 @@
 // steps end 0.2 to 0.65 times as far from a long double run as with FP64 arithmetic (over
 // spacings 0.0245-0.6, time steps 1e-7 to 1e-3, tau 1-3, means 0 and 2).
 // About 370 instructions per site instead of 29 FP64 ones: the plain kernel on the
-// 4096-lattice ensemble went from 1.90e10 to 3.5e10 site-updates/s.  What bounds it now is
-// the integer pipe (ALU 54 % busy) and the conversions (FP64 pipe 55 %).
+// 4096-lattice ensemble went from 1.90e10 to 3.5e10 site-updates/s.  What bounds the many-step
+// kernel (4.5e10) now is the integer pipe (ALU 55 % busy) and the conversions (FP64 pipe 56 %).
 #pragma once
 
 #include <cstdint>

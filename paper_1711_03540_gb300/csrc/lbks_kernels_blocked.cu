@@ -23,11 +23,12 @@
 // 1.12 us; 2^20 sites 3.1 against 2.2 us, so large FP32 batches stay register-resident.
 // Not for scaled FP16, whose results depend on where launches end (rounded there).
 // Per step and stretch: the halos cost 2 c_max k of NT sites, a launch 1.5 to 2 us in all.
-// Measured (GB300): one 4096-site D1Q7 FP64 lattice 16.8 -> 0.75 us per step (stretches of
+// Measured (GB300): one 4096-site D1Q7 FP64 lattice 16.8 -> 0.71 us per step (stretches of
 // 32 sites, 16 steps per launch; bound by the latency of one warp's collision), the
-// 4096-lattice FP64 ensemble 615 -> 219 us per step, 4.3e10 site-updates/s (256 threads, 4
-// steps per launch; bound by the integer pipe, 54 % busy, and the conversions, 56 %), 122
-// front lattices 9.3 -> 2.3 us per step, 24 FP32 lattices 0.87 -> 0.37 us per step.
+// 4096-lattice FP64 ensemble 615 -> 209 us per step, 4.5e10 site-updates/s (128 threads, 2
+// steps per launch; bound by the integer pipe, 55 % busy, and the conversions, 56 %, which
+// contend; having L2 fetch the state a round of blocks ahead gave 0.6 %), 122 front lattices
+// 10.5 -> 2.9 us per step, 24 FP32 lattices 0.87 -> 0.37 us per step.
 #include "lbks_collapse.cuh"
 #include "lbks_device.cuh"
 #include "lbks_plan.h"
@@ -145,9 +146,9 @@ __global__ void __launch_bounds__(NTM, MINB)
 // (the fixed nodes keep their values, put in both parities once).  Z: the operations that
 // add zero are left out (collapse_site's ZB, and ZR in FP64).  FP64 is bound by the
 // FP64 pipe, so what counts is to use every SM's: one 4096-site lattice 25 -> 1.0 us per
-// step, 24 lattices 25 -> 3.9, the 4096-lattice ensemble 442 -> 418; FP32, 24 lattices: 1.02
-// -> 0.34 us, one lattice 0.57 -> 0.20 (300 lattices: 1.03 either way, so larger batches
-// stay register-resident).
+// step (0.85 with Z), 24 lattices 25 -> 3.9 (2.9), the 4096-lattice ensemble 442 -> 418 (303);
+// FP32, 24 lattices: 1.02 -> 0.34 us (0.31), one lattice 0.57 -> 0.20 (300 lattices: 1.03
+// either way, so larger batches stay register-resident).
 template <int C, int ST, bool RES, bool ONE, bool Z>
 __global__ void __launch_bounds__(512, 2)
     blocked_collapse_kernel(Arena src, Arena dst, const RunDesc* __restrict__ runs, const Piece* __restrict__ pieces,
