@@ -274,9 +274,9 @@ LB_KS_API int64_t lb_ks_steps_done(const lb_ks_t *h);
 /*
  * Describe the handle: kernel family actually used (LB_KS_KERNEL_*), resident
  * sites per thread (1: the one-site-per-thread resident kernel, the automatic choice for
- * F64 and for F32 batches too small to fill the device), threads per block, steps per launch and blocks per work group
- * of whole lattices (1 or 2; all 0 when not resident), number of runs and total
- * sites.  Any pointer may be NULL.
+ * F64 and for F32 batches too small to fill the device), threads per block, steps per launch
+ * and blocks per work group of whole lattices (1 or 2, with one site per thread up to 8; all 0
+ * when not resident), number of runs and total sites.  Any pointer may be NULL.
  */
 LB_KS_API int lb_ks_describe(const lb_ks_t *h, int *kernel, int *sites_per_thread, int *threads_per_block,
                    int *steps_per_launch, int *cluster_size, int32_t *nruns, int64_t *total_sites);
@@ -285,7 +285,8 @@ LB_KS_API int lb_ks_describe(const lb_ks_t *h, int *kernel, int *sites_per_threa
  * The register-resident plan of the handle (no counterpart in the paper): the work
  * lists ("lanes") that run concurrently, one record of LB_KS_LANE_FIELDS int32 per
  * lane written to lanes[8 * l .. 8 * l + 7] for l < max_lanes:
- *   [0] blocks per work group (1, or 2 for a thread block cluster pair)
+ *   [0] blocks per work group (1, or 2 for a thread block cluster pair; one site per thread: up
+ *       to 8, and [2] then counts the bundles of single blocks)
  *   [1] work groups launched (persistent grid)
  *   [2] bundles (work items of packed lattices) in the lane's queue
  *   [3] steps per launch

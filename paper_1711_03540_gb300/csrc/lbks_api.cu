@@ -340,14 +340,33 @@ cudaError_t prepared(int kind, int Q, int prec, int S, int NT, bool zb, int* out
   return cudaSuccess;
 }
 
-// Plan of the blocked kernel (one site per thread), if its step is estimated to take less
-// than `than` microseconds: LB_KS_OK, 1 if not, or an error.
+// Plan of the blocked kernel (one site per thread), lattices over the blocks of a cluster or in
+// haloed stretches, if its step is estimated to take less than `than` microseconds: LB_KS_OK, 1 if not, or an error.
 int setup_blocked(lb_ks* h, int sms, double than) {
   const int R = h->opts.recentre_every;
-  const BlockedTiling b = choose_blocked(h->N, h->reservoir, h->Q, blocked_cost(h->Q, h->prec == kF64, h->nplanes == 1),
-                                         sms, R > 0 ? std::min(R, 1000) : 1000);
-  if (b.NT == 0 || b.us >= than) return 1;
+  const int kwhole = R > 0 ? std::min(R, 1000) : 1000;
+  const BlockedCost cost = blocked_cost(h->Q, h->prec == kF64, h->nplanes == 1);
+  const BlockedTiling b = choose_blocked(h->N, h->reservoir, h->Q, cost, sms, kwhole);
   std::vector<Piece> pieces;
+  if (h->prec == kF64 && h->nplanes > 1) {
+    const ClusterTiling c = choose_clusters(h->N, h->reservoir, h->Q, sms, kwhole);
+    std::vector<int2> bundles;
+    if (c.us < 0.92 * std::min(b.us, than) && plan_clusters(h->N, h->reservoir, h->cmax, c.NT, c.CL, &pieces, &bundles)) {
+      Lane& L = h->lanes[0];
+      int rc;
+      if ((rc = upload_lane(h, &L, pieces, bundles, c.CL, kwhole, false, 1.0))) return rc;
+      L.grid = L.nbundles / c.CL;
+      L.one = L.spread = false;
+      h->nlanes = 1;
+      h->blocked = true;
+      h->S = 1;
+      h->NT = c.NT;
+      h->kmax = kwhole;
+      h->kseg = 1;
+      return LB_KS_OK;
+    }
+  }
+  if (b.NT == 0 || b.us >= than) return 1;
   if (!plan_blocked(h->N, h->reservoir, h->cmax, b.NT, b.k, &pieces)) return 1;
   bool segmented = false;
   for (const Piece& p : pieces) segmented = segmented || p.st_hi - p.st_lo < p.n;

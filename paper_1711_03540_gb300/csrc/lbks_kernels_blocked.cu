@@ -28,7 +28,7 @@
 // 4096-lattice FP64 ensemble 615 -> 209 us per step, 4.5e10 site-updates/s (128 threads, 2
 // steps per launch; bound by the integer pipe, 55 % busy, and the conversions, 56 %, which
 // contend; having L2 fetch the state a round of blocks ahead gave 0.6 %), 122 front lattices
-// 10.5 -> 2.9 us per step, 24 FP32 lattices 0.87 -> 0.37 us per step.
+// 9.8 -> 2.2 us per step (over clusters; stretches 2.9), 24 FP32 lattices 0.87 -> 0.37 us per step.
 #include "lbks_collapse.cuh"
 #include "lbks_device.cuh"
 #include "lbks_plan.h"
@@ -45,6 +45,19 @@ using plan::kBlockedPieces;
 // 3.4 instead of 2.4 us per step); at the last step, a small batch waits for the launch.
 constexpr int kNextGrid = 2;
 
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void store_cluster(uint32_t addr, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // NTM: the most threads a block of this instance has.
 template <int Q, int ST, int NTM> struct BlockedCfg {
   // Row of the exchange area, a compile-time stride: a column per thread.  FP64: and, for
@@ -60,7 +73,15 @@ template <int Q, int ST, int NTM> struct BlockedCfg {
 // register budget: 80 in FP64 (24 warps), 64 in FP32 where SMs are to be filled; FP64 batches
 // of at most a block per SM take what the compiler wants instead (122), which shortens the
 // one warp per scheduler's chain by 4 to 6 %.
-template <int Q, int ST, int NTM, int MINB, bool RES, bool ONE>
+// CLU: the blocks of a cluster hold lattices together (plan_clusters), without halos: a portion's
+// edge values are also stored into the guard columns of the block that holds its neighbour
+// (st.shared::cluster; the portion itself where a lattice lies in one block), and the step's barrier is
+// the cluster's.  For FP64 batches with lattices longer than a block: their stretches cost up
+// to two thirds more sites in halos, and launches that end block by block every 4 to 16
+// steps.  The cluster barrier adds 0.3 us to a step's latency (1.02 against 0.72 us with one
+// block an SM), which other blocks of the SM cover; 122 front lattices 2.86 -> 2.23 us per
+// step, 140 lattices of up to 1200 sites 3.55 -> 2.27 us, single lattices stay in stretches.
+template <int Q, int ST, int NTM, int MINB, bool RES, bool ONE, bool CLU = false>
 __global__ void __launch_bounds__(NTM, MINB)
     blocked_step_kernel(Arena src, Arena dst, const RunDesc* __restrict__ runs, const Piece* __restrict__ pieces,
                         const int2* __restrict__ bundles, int ksteps) {
@@ -81,7 +102,7 @@ __global__ void __launch_bounds__(NTM, MINB)
   }
   const Piece pc = pieces[p];
   const int n = pc.n, j = t - pc.t0;
-  const bool active = j < n;
+  const bool active = j < n && (!CLU || bundles[blockIdx.x].y > 0);
   wait_prior_grid();
   const RunDesc& d = runs[pc.run];
   int x = (int)pc.x0 + j;  // run-local site (N <= 2^30)
@@ -102,6 +123,13 @@ __global__ void __launch_bounds__(NTM, MINB)
     const int c = (i + 1) / 2;
     from[i] = (i & 1) ? (j >= c ? -c : n - c) : (j + c < n ? c : c - n);
   }
+  uint32_t edge = 0;  // where this thread's values that leave the portion go, in the cluster's shared memory
+  if constexpr (CLU) {
+    const bool right = j >= n - C;
+    const int to = right ? pc.pad_ : pc.halo;
+    edge = map_to_rank(smem_addr(&ex[0][0][(to & 0xffff) + (right ? j - n : j)]), (uint32_t)to >> 16);
+    cluster_barrier();  // every block runs before another writes into it
+  }
   for (int s = 0; s < ksteps; ++s) {
     if (s == ksteps - kNextGrid || (s == 0 && ksteps < kNextGrid)) allow_next_grid();
     CT* const xs = own + (s & 1) * (Q - 1) * XS;
@@ -113,7 +141,12 @@ __global__ void __launch_bounds__(NTM, MINB)
         CT* const w = xs + (i - 1) * XS;
         *w = g[i];
         // the last c sites' right-moving values enter at the piece's start, and so on
-        if (kGuard && ((i & 1) ? j >= n - c : j < c)) w[(i & 1) ? -n : n] = g[i];
+        if (kGuard && ((i & 1) ? j >= n - c : j < c)) {
+          if constexpr (CLU)
+            store_cluster(edge + (uint32_t)((((s & 1) * (Q - 1) + i - 1) * XS) * sizeof(CT)), g[i]);
+          else
+            w[(i & 1) ? -n : n] = g[i];
+        }
       }
       if constexpr (RES) {
         if (fixed) {
@@ -127,7 +160,9 @@ __global__ void __launch_bounds__(NTM, MINB)
         }
       }
     }
-    __syncthreads();
+    // (double-buffered: a block writes parity s again only after all have passed s + 1's)
+    if constexpr (CLU) cluster_barrier();
+    else __syncthreads();
     if (active && !fixed) {
 #pragma unroll
       for (int i = 1; i < Q; ++i) g[i] = xs[(i - 1) * XS + (kGuard ? -speed(i) : from[i])];
@@ -229,6 +264,30 @@ cudaError_t launch_t(const ResidentLaunch& L, cudaStream_t s) {
   }
 }
 
+template <int Q, bool RES, int NTM>
+cudaError_t launch_cluster_n(const ResidentLaunch& L, cudaStream_t s) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)L.nbundles);
+  cfg.blockDim = dim3((unsigned)L.NT);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)L.cl;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, blocked_step_kernel<Q, kF64, NTM, 768 / NTM, RES, false, true>, L.src, L.dst, L.runs,
+                            L.pieces, L.bundles, L.ksteps);
+}
+
+template <int Q, bool RES>
+cudaError_t launch_cluster_t(const ResidentLaunch& L, cudaStream_t s) {
+  if (L.storage != kF64 || L.one || L.nbundles % L.cl || L.cl > 8 || L.NT > 384) return cudaErrorInvalidValue;
+  if (L.NT <= 128) return launch_cluster_n<Q, RES, 128>(L, s);
+  if (L.NT <= 256) return launch_cluster_n<Q, RES, 256>(L, s);
+  return launch_cluster_n<Q, RES, 384>(L, s);
+}
+
 template <int Q, int ST, bool RES, bool Z>
 cudaError_t launch_collapse_z(const ResidentLaunch& L, cudaStream_t s) {
   constexpr int C = cmax_of(Q);
@@ -268,6 +327,10 @@ cudaError_t launch_blocked(const ResidentLaunch& L, bool reservoir, cudaStream_t
     return cudaErrorInvalidValue;
   }
   if (L.NT > (storage == kF64 ? 384 : 512)) return cudaErrorInvalidValue;
+  if (L.cl > 1) {
+    if (Q == 5) return reservoir ? launch_cluster_t<5, true>(L, s) : launch_cluster_t<5, false>(L, s);
+    return reservoir ? launch_cluster_t<7, true>(L, s) : launch_cluster_t<7, false>(L, s);
+  }
   if (reservoir) LBKS_BLOCKED_DISPATCH(return (launch_t<Qc, STc, true>(L, s)));
   else LBKS_BLOCKED_DISPATCH(return (launch_t<Qc, STc, false>(L, s)));
   return cudaErrorInvalidValue;

@@ -330,15 +330,20 @@ struct Bins {
     for (int i : mem) link(b, i);
     fix(b);
   }
+  // The first group with `need` threads free; groups() if none has.
+  size_t first_with(int need) const {
+    if (tn == 0 || tree[1] < need) return groups();
+    size_t p = 1;
+    while (p < tn) p = tree[2 * p] >= need ? 2 * p : 2 * p + 1;
+    return p - tn;
+  }
   // First fit: the first group with room for the piece.  A piece never spans the
   // block edge of a pair work group here: it goes into block 0's free threads or
   // after block 1's taken ones.
   bool first_fit(std::vector<Piece>& pieces, int i) {
     const int need = pieces[i].nthr;
-    if (tn == 0 || tree[1] < need) return false;
-    size_t p = 1;
-    while (p < tn) p = tree[2 * p] >= need ? 2 * p : 2 * p + 1;
-    const size_t b = p - tn;
+    const size_t b = first_with(need);
+    if (b == groups()) return false;
     if (pair && used0[b] + need <= cap / 2) {
       pieces[i].t0 = used0[b];
       used0[b] += need;
@@ -372,6 +377,141 @@ inline std::vector<int> by_threads_desc(const std::vector<Piece>& pieces) {
   std::vector<int> nthr(pieces.size());
   for (size_t i = 0; i < pieces.size(); ++i) nthr[i] = pieces[i].nthr;
   return stable_desc(nthr);
+}
+
+// ---- one site per thread over the blocks of a cluster: a lattice's sites lie on consecutive
+// threads of the cluster's CL blocks of NT threads, cut into portions at block edges, with no
+// halos (a portion's edge values go straight into the blocks that hold its neighbours).
+
+// The fewest threads a portion takes: its two edges are apart, and a block holds at most
+// kBlockedPieces portions.
+inline int portion_min(int C, int NT) { return std::max(2 * C, NT / kBlockedPieces); }
+
+// Places n sites on a cluster whose threads before pos are taken, in portions (pos, length)
+// that each lie in one block; returns the position after them.
+template <typename F>
+inline int64_t place_portions(int64_t pos, int64_t n, int C, int NT, F portion) {
+  const int64_t pmin = portion_min(C, NT);
+  int64_t room = NT - pos % NT;
+  if (std::max(n, pmin) > room && (room < 2 * pmin || n < 2 * pmin)) {  // no cut leaves two portions
+    pos += room;
+    room = NT;
+  }
+  for (;;) {
+    int64_t len = std::min(n, room);
+    if (n > len && n - len < pmin) len = n - pmin;
+    portion(pos, len);
+    n -= len;
+    if (n == 0) return pos + std::max(len, pmin);
+    pos += room;  // (shortened portions leave threads idle)
+    room = NT;
+  }
+}
+
+// Pieces (portions) and bundles (one per block, CL consecutive ones a cluster; possibly empty)
+// of lattices packed first fit, longest first.  A piece's halo and pad_ say where its edge
+// values go: block of the cluster << 16 | column of that block's exchange area, of the left
+// neighbour's right guard and of the right neighbour's first site.  False if some lattice does
+// not fit a cluster.
+inline bool plan_clusters(const std::vector<int64_t>& Ns, bool reservoir, int C, int NT, int CL,
+                          std::vector<Piece>* pieces, std::vector<int2>* bundles) {
+  pieces->clear();
+  bundles->clear();
+  const int64_t ghost = reservoir ? C : 0, cap = (int64_t)CL * NT, pmin = portion_min(C, NT);
+  std::vector<int> order(Ns.size());
+  for (size_t r = 0; r < Ns.size(); ++r) order[r] = (int)r;
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return Ns[(size_t)a] > Ns[(size_t)b]; });
+  Bins cl;  // used: a cluster's threads before its free ones
+  cl.cap = (int)cap;
+  std::vector<int> in_block;                    // portions in the block that the last taken thread lies in
+  std::vector<std::pair<int64_t, Piece>> held;  // (block, portion)
+  const auto end = [&](int64_t pos, int64_t n) { return place_portions(pos, n, C, NT, [](int64_t, int64_t) {}); };
+  for (int r : order) {
+    const int64_t n = Ns[(size_t)r] + 2 * ghost;
+    if (n > cap) return false;
+    size_t b = cl.first_with((int)n);
+    if (b < cl.groups() && end(cl.used[b], n) > cap) b = cl.first_with((int)(n + 2 * pmin));
+    if (b == cl.groups() || end(cl.used[b], n) > cap) {
+      if (end(0, n) > cap) return false;
+      b = cl.new_group(0, 0);
+      in_block.push_back(0);
+    }
+    const size_t from = held.size();
+    int64_t x = -ghost, block = cl.used[b] > 0 ? (cl.used[b] - 1) / NT : 0;
+    cl.used[b] = (int)place_portions(cl.used[b], n, C, NT, [&](int64_t pos, int64_t len) {
+      if (pos / NT != block) in_block[b] = 0;
+      block = pos / NT;
+      Piece p{};
+      p.run = r; p.t0 = (int)(pos % NT); p.n = (int)len; p.nthr = (int)std::max(len, pmin); p.x0 = x; p.st_hi = p.n;
+      p.pad_ = (int)((block << 16) | (p.t0 + C * (2 * in_block[b] + 1)));  // (its own first column, for now)
+      ++in_block[b];
+      x += len;
+      held.emplace_back((int64_t)b * CL + block, p);
+    });
+    const size_t m = held.size() - from;
+    std::vector<int32_t> own(m);
+    for (size_t q = 0; q < m; ++q) own[q] = held[from + q].second.pad_;
+    for (size_t q = 0; q < m; ++q) {
+      const size_t l = (q + m - 1) % m;
+      held[from + q].second.halo = own[l] + held[from + l].second.n;
+      held[from + q].second.pad_ = own[(q + 1) % m];
+    }
+    cl.fix(b);
+  }
+  std::stable_sort(held.begin(), held.end(), [](const auto& a, const auto& b) { return a.first < b.first; });
+  bundles->assign(cl.groups() * (size_t)CL, int2{0, 0});
+  for (const auto& [block, p] : held) {
+    int2& bd = (*bundles)[(size_t)block];
+    if (bd.y++ == 0) bd.x = (int)pieces->size();
+    pieces->push_back(p);
+  }
+  return true;
+}
+
+struct ClusterTiling {
+  int NT = 0, CL = 0;
+  double us = 1e300;
+};
+
+// The cheapest cluster tiling for FP64 batches with lattices too long for a block.  No halos and
+// no launch ends, but a cluster barrier per step: measured (GB300, D1Q7, 128-thread blocks) 1.02,
+// 1.30, 1.53, 1.84, 2.20, 2.55 us per step with 1 to 6 blocks an SM, t0 + t1 w for w warps.
+// Clusters fill the SMs a little unevenly (144 blocks put two on some of 152 SMs), and blocks
+// beyond 768 threads an SM run all their steps after the others.  Large clusters wait for
+// room for all their blocks (8 x 384: up to 1.7 times the model, not considered; 8 x 256: 1.05
+// to 1.2, and no more than 0.85 of the device at once).  The caller asks for 8 % less than the
+// launches' estimate: over 200 batches of 4 to 1400 lattices of 200 to 2900 sites it gave 1.02
+// to 1.56 times their rate where clusters were chosen (front tests of 122 lattices: D1Q7
+// 2.86 -> 2.23 us per step, D1Q5 2.01 -> 1.41).
+inline ClusterTiling choose_clusters(const std::vector<int64_t>& Ns, bool reservoir, int Q, int sms, int kwhole) {
+  const double t0 = Q == 7 ? 0.70 : 0.58, t1 = Q == 7 ? 0.08 : 0.058;
+  const int C = (Q - 1) / 2;
+  const size_t stride = (Ns.size() + 127) / 128;
+  std::vector<int64_t> n;
+  for (size_t r = 0; r < Ns.size(); r += stride) n.push_back(Ns[r] + (reservoir ? 2 * C : 0));
+  std::sort(n.begin(), n.end(), std::greater<int64_t>());
+  const int64_t longest = *std::max_element(Ns.begin(), Ns.end()) + (reservoir ? 2 * C : 0);
+  ClusterTiling best;
+  for (int CL : {2, 4, 8})
+    for (int NT : {64, 96, 128, 192, 256, 384}) {
+      const int64_t pmin = portion_min(C, NT), cap = (int64_t)CL * NT;
+      if (longest <= NT || longest + 2 * pmin > cap || cap > 2048) continue;
+      std::vector<int64_t> room;
+      for (int64_t v : n) {
+        size_t b = 0;
+        while (b < room.size() && room[b] < v) ++b;
+        if (b == room.size()) room.push_back(cap);
+        room[b] -= std::max(v, pmin) + (v > NT ? pmin : pmin / 2);
+      }
+      const double blocks = (double)(room.size() * stride) * CL, per = (double)(768 / NT);
+      const double even = 0.95 * sms, hold = per * (cap > 1536 ? 0.85 : 0.95) * sms, full = std::floor(blocks / hold);
+      const double rest = std::ceil((blocks - full * hold) / even - 1e-9);
+      const double slow = cap > 1536 ? 1.15 : NT > 256 ? 1.08 : 1.0;
+      const auto step = [&](double b) { return slow * (t0 + t1 * std::max(b * NT / 32.0, 4.0)); };
+      const double us = full * step(per) + (rest > 0.0 ? step(rest) : 0.0) + 4.0 / kwhole;  // (a launch)
+      if (us < best.us) best = ClusterTiling{NT, CL, us};
+    }
+  return best;
 }
 
 // Time of a step of the register-resident kernel (D1Q7, microseconds), S sites per thread
