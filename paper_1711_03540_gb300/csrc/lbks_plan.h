@@ -528,7 +528,7 @@ inline double resident_step_us(int S, int NT, int q, bool pairs) {
     case 20: return at(0.48, 0.35);
     case 18: return at(0.385, 0.32);
     case 16: return at(0.345, 0.225);
-    case 8: return at(0.285, 0.145);
+    case 8: return at(0.285, 0.165);
     case 6: return at(0.26, 0.105);
     case 4: return at(0.235, 0.09);
     default: return 0.0;
@@ -544,6 +544,7 @@ struct ResidentTiling {
   double us = 1e300;
 };
 
+// (D1Q5: 0.7 of these times at 20 sites, 0.84 at fewer.)
 // The estimate for one tiling of which `bps` blocks fit an SM: blocks run in rounds of
 // sms bps, each as long as a full SM's step, so a batch of 1.7 rounds takes as long as
 // one of 2, and smaller blocks that need 2 shorter rounds are faster; a batch of less
@@ -556,21 +557,32 @@ inline ResidentTiling rate_resident(const std::vector<int64_t>& Ns, int Q, int S
   const double edge = S == 18 ? 14.5 : 20.0;
   constexpr double kLaunchUs = 3.0, kRingCost = 1.4, kRingUs = 0.4;
   const int C = (Q - 1) / 2, h = C * kPairStepsMax;
-  const double scale = Q == 7 ? 1.0 : 0.7;
+  const double scale = Q == 7 ? 1.0 : (S == 20 ? 0.7 : 0.84);
   ResidentTiling t;
   t.S = S;
   t.NT = NT;
-  const size_t stride = (Ns.size() + 127) / 128;  // a sample of a large batch
-  std::vector<int> threads;  // of whole lattices and halves
-  int64_t halves = 0, rings = 0;
+  const size_t stride = (Ns.size() + 127) / 128;  // a sample of a large batch is packed
+  std::vector<int> threads;  // of the sample's whole lattices and halves
+  double all = 0.0, sampled = 0.0;  // their sum over the batch and the sample
+  int64_t whole = 0, halves = 0, rings = 0;
   std::vector<int64_t> cut;
-  for (size_t r = 0; r < Ns.size(); r += stride) {
-    const int64_t v = (Ns[r] + S - 1) / S, half = ((Ns[r] + 1) / 2 + 2 * h + S - 1) / S + 1;
-    if (v <= NT) {
-      threads.push_back((int)v);
-    } else if (half <= NT) {
-      threads.insert(threads.end(), 2, (int)half);
-      halves += 2;
+  for (size_t r = 0; r < Ns.size(); ++r) {
+    int64_t v = (Ns[r] + S - 1) / S;  // (copies of lattices that do not split into S and S - 1, as in plan_pieces)
+    for (int64_t n = Ns[r]; n <= v * (S - 1) && v <= 2 * NT;) {
+      n += Ns[r];
+      v = (n + S - 1) / S;
+    }
+    const int64_t half = ((Ns[r] + 1) / 2 + 2 * h + S - 1) / S + 1;
+    const bool in = r % stride == 0;
+    if (v <= NT || half <= NT) {
+      const int held = (int)(v <= NT ? v : half), n = v <= NT ? 1 : 2;
+      all += (double)held * n;
+      whole += n;
+      halves += n == 2 ? 2 : 0;
+      if (in) {
+        threads.insert(threads.end(), (size_t)n, held);
+        sampled += (double)held * n;
+      }
     } else if (v <= 2 * NT) {  // one ring across a pair waits on the other block every step
       if (!kfix) return t;     // (the fixed tiling's estimate is still wanted)
       ++rings;
@@ -579,7 +591,8 @@ inline ResidentTiling rate_resident(const std::vector<int64_t>& Ns, int Q, int S
     }
   }
   const bool pairs = halves + rings > 0;
-  const double pieces = (double)(threads.size() + rings) * (double)stride;
+  if (pairs && S <= 8 && !kfix) return t;  // (the cluster kernel's time with these is 1.8 times a block's)
+  const double pieces = (double)(whole + rings);
   // first fit, largest first: the blocks they fill
   std::sort(threads.begin(), threads.end(), std::greater<int>());
   const int64_t widest = pairs ? NT : (threads.empty() ? 0 : threads.front());
@@ -590,7 +603,13 @@ inline ResidentTiling rate_resident(const std::vector<int64_t>& Ns, int Q, int S
     if (b == room.size()) room.push_back(NT);
     room[b] -= v;
   }
-  const double blocks = ((double)room.size() + 2.0 * kRingCost * (double)rings) * (double)stride;
+  double blocks = (double)room.size();
+  if (stride > 1 && !room.empty()) {  // as full as the sample's, without its emptiest
+    const double most = *std::max_element(room.begin(), room.end());
+    const double n = (double)room.size(), fill = n > 1.0 ? (sampled - (NT - most)) / (n - 1.0) : (double)NT;
+    blocks = all / fill;
+  }
+  blocks += 2.0 * kRingCost * (double)rings;
   const double slots = (double)sms * bps;
   const auto warps = [&](double per_sm, int64_t threads) {  // per scheduler: a block's first warp is the first's
     return (int)std::ceil(per_sm - 1e-9) * (int)((threads + 127) / 128);
@@ -614,7 +633,7 @@ inline ResidentTiling rate_resident(const std::vector<int64_t>& Ns, int Q, int S
       if (room <= 0) break;
       double n = 0.0;
       for (int64_t N : cut) n += (double)((N + room - 1) / room);
-      const double rounds = std::ceil(n * (double)stride / slots);
+      const double rounds = std::ceil(n / slots);
       const double c = rounds * (full + edge / k) + kLaunchUs / k;
       if (c < best) { best = c; t.kseg = k; }
       if (kfix) break;

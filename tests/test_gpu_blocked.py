@@ -97,7 +97,7 @@ def test_reservoir_ends_match_oracle(lb, Q, runs):
 @pytest.mark.parametrize("prec", [1, 2])
 @pytest.mark.parametrize("nruns,nmin,nmax", [(1, 1000, 1000), (4, 500, 2700), (24, 256, 8192), (60, 100, 600),
                                              (238, 164, 549), (354, 548, 1770), (1024, 64, 256), (2500, 100, 700),
-                                             (1024, 220, 4000), (3, 9000, 11000)])
+                                             (1024, 220, 4000), (3, 9000, 11000), (1187, 18, 6303), (1187, 16, 3000)])
 def test_tiling_chosen_by_size_equals_the_fixed_one(lb, prec, nruns, nmin, nmax):
     """FP32 and scaled FP16 (rounded at launch edges, which the choice must not move): the
     default plan's results are those of 20 sites x 256 threads, bitwise."""
