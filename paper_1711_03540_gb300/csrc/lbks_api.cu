@@ -427,11 +427,16 @@ int setup_resident(lb_ks* h, bool required, int S_force = 0, int NT_force = 0, d
   const int R = h->opts.recentre_every;
   ResidentTiling fixed;  // S = 0: the first tiling below that holds the lattices
   if (col && S_force == 0 && free_tiling(h)) {
-    // FP32: a step of the register-resident collapse takes about 1 us a round of its
-    // 8192-site blocks; FP64: 28 us a round of 4096 sites, bound by the FP64 pipe as the
-    // blocked collapse is, which spreads over the SMs and cuts no lattice into few blocks
-    const double us = (h->Q == 7 ? 1.0 : 0.75) * std::max(1.0, 1.03 * (double)h->total_sites / (8192.0 * sms));
-    if ((rc = setup_blocked(h, sms, h->prec == kF64 ? 1e300 : 0.95 * us)) <= 0) return rc;
+    // FP64: the register-resident collapse takes 28 us a round of 4096 sites, bound by the FP64
+    // pipe as the blocked collapse is, which spreads over the SMs and cuts no lattice into few
+    // blocks
+    double us = 1e300;
+    if (h->prec == kF32) {
+      fixed = choose_collapse(h->N, sms);
+      const double scale = h->Q == 5 ? 0.84 : h->zb ? 1.0 : 1.15;
+      us = 0.95 * scale * (fixed.S ? fixed.us : std::max(1.0, (double)h->total_sites / (8192.0 * sms)));
+    }
+    if ((rc = setup_blocked(h, sms, us)) <= 0) return rc;
   }
   if (!col && S_force == 0 && free_tiling(h)) {
     if (h->prec != kF64)
@@ -448,7 +453,8 @@ int setup_resident(lb_ks* h, bool required, int S_force = 0, int NT_force = 0, d
   if (fixed.S) cand.push_back(fixed.S);
   if (S_force) cand.push_back(S_force);
   else if (h->opts.sites_per_thread) cand.push_back(h->opts.sites_per_thread);
-  else if (col) cand = h->prec == kF64 ? std::vector<int>{16, 8} : std::vector<int>{32, 16, 8};
+  else if (col && h->prec == kF64) cand = {16, 8};
+  else if (col) cand.insert(cand.end(), {32, 16, 8});
   else if (h->prec == kF64) cand = {8, 6, 4};
   else cand.insert(cand.end(), {20, 18, 12, 8, 16, 6, 4});
   for (size_t c = 0; c < cand.size(); ++c) {

@@ -671,6 +671,60 @@ ResidentTiling choose_resident(const std::vector<int64_t>& Ns, int Q, bool f16, 
   return best;
 }
 
+// The register-resident tau = 1 collapse's tiling (FP32).  Step times by blocks per SM, measured
+// (GB300, D1Q7 without the terms that add zero; other runs scale them together): 32 sites x 256
+// threads 0.865 with one and 1.59 us with two, 32 x 384 1.25, 16 x 384 0.68, 16 x 256 0.51,
+// 8 x 384 0.41.  Lattices shorter than S (S - 1) are held as copies, so
+// short ones want few sites per thread; a batch of 1.1 to 1.4 rounds of 8192 sites wants
+// 32 x 384 (700 lattices of 256 to 8192 sites: 1.59 -> 1.26 us), one of 0.3 rounds 8 x 384 (101
+// lattices of 1504 to 3031 sites: 0.86 -> 0.41 us).  32 x 256 stays unless another
+// is estimated 8 % faster.  us is the chosen one's estimate.
+inline ResidentTiling choose_collapse(const std::vector<int64_t>& Ns, int sms) {
+  struct Cost { int S, NT; double first, more; };  // us with one block an SM, and for each further one
+  ResidentTiling best;
+  const size_t stride = (Ns.size() + 255) / 256;
+  for (const Cost c : {Cost{32, 256, 0.865, 0.725}, Cost{32, 384, 1.25, 1.25}, Cost{16, 384, 0.69, 0.69},
+                       Cost{16, 256, 0.51, 0.51}, Cost{8, 384, 0.41, 0.41}}) {
+    std::vector<int> threads;
+    double all = 0.0, sampled = 0.0;
+    bool whole = true;
+    for (size_t r = 0; r < Ns.size() && whole; ++r) {
+      int64_t v = (Ns[r] + c.S - 1) / c.S;
+      for (int64_t n = Ns[r]; n <= v * (c.S - 1) && v <= c.NT;) {
+        n += Ns[r];
+        v = (n + c.S - 1) / c.S;
+      }
+      whole = v <= c.NT;
+      all += (double)v;
+      if (r % stride == 0) {
+        threads.push_back((int)v);
+        sampled += (double)v;
+      }
+    }
+    if (!whole) continue;
+    std::sort(threads.begin(), threads.end(), std::greater<int>());
+    std::vector<int> room;
+    for (int v : threads) {
+      size_t b = 0;
+      while (b < room.size() && room[b] < v) ++b;
+      if (b == room.size()) room.push_back(c.NT);
+      room[b] -= v;
+    }
+    double blocks = (double)room.size();
+    if (stride > 1) {  // as full as the sample's, without its emptiest; 2 % for what it misses
+      const double most = *std::max_element(room.begin(), room.end());
+      blocks = 1.02 * all / (blocks > 1.0 ? (sampled - (c.NT - most)) / (blocks - 1.0) : (double)c.NT);
+    }
+    const double us = c.first + c.more * (std::max(1.0, std::ceil(blocks / sms - 1e-9)) - 1.0);
+    if (best.S == 0 || us < std::min(best.us, best.S == 32 && best.NT == 256 ? 0.92 * best.us : best.us)) {
+      best.S = c.S;
+      best.NT = c.NT;
+      best.us = us;
+    }
+  }
+  return best;
+}
+
 // First-fit decreasing packing of whole lattices: a lattice held as two halves opens a
 // cluster pair (one half at the start of each block), one longer than one block (more
 // than NT threads) opens a pair as a ring across both blocks; the others fill the
