@@ -90,10 +90,14 @@ LBKS_HD uint32_t hi32(uint64_t x) { return (uint32_t)(x >> 32); }
 // A value on the site's grid: |g| <= 2^(e - 1022), as h 2^28 + l in units of 2^(e - 1078)
 // (both limbs carry the sign sg), a lost bit jammed into l.
 LBKS_HD void to_limbs(uint64_t bits, uint32_t e, int32_t& h, int32_t& l, int32_t& sg) {
-  const uint32_t hi = hi32(bits), lo = (uint32_t)bits;
-  const uint32_t ei = (hi & 0x7fffffffu) >> 20;
+  const uint32_t hi = hi32(bits), lo = (uint32_t)bits, mag = hi & 0x7fffffffu;
+  const uint32_t ei = mag >> 20;
   const uint64_t p = (bits << 11) | ((uint64_t)0x80000000u << 32);   // mantissa, leading bit at 63
-  const uint32_t rest = shl32(lo, ei + (35u - e));                   // the bits below the grid
+  // the bits below the grid: of the low word alone down to 35 binades, then of all of the
+  // mantissa, and from 56 on the leading one too, which every value but zero has
+  const uint32_t n = e - ei;
+  uint32_t rest = shl32(lo, 35u - n);
+  if (n > 35u) rest = n > 55u ? mag : lo | shl32(hi, 67u - n);
   sg = ((int32_t)hi >> 31) | 1;
   h = (int32_t)shr32(hi32(p), (e + 4u) - ei) * sg;
   l = (int32_t)(((uint32_t)shr64(p, (e + 8u) - ei) & (uint32_t)kMask) | (rest < 1u ? rest : 1u)) * sg;
