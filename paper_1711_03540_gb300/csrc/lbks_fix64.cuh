@@ -13,8 +13,7 @@
 //     conserved mass linearly in time instead of as a random walk.
 //  2. s = sum g_i is exact on the grid; r g_i + a_i s + b_i s^2 are sums of limb products
 //     (32 x 32 -> 64-bit multiply-adds), on a grid of 2^(e - 1079).  The products of two low
-//     limbs are left out; their mean, where it is not zero, is added (constants with a_p,
-//     the sign of g_i with r).
+//     limbs are left out; their mean, where it is not zero, is added (the sign of g_i with r).
 //  3. g_0 takes s minus the others, in integers: the collision keeps mass to the conversions.
 //  4. The hardware's conversion (64-bit integer to FP64, round to nearest even, on the idle
 //     FP64 pipe) rounds each result once.
@@ -143,8 +142,11 @@ LBKS_HD bool fix_collide(const uint64_t (&g)[Q], uint64_t (&out)[Q], const FixCo
   int32_t sh = h[0], sl = l[0];
   LBKS_UNROLL
   for (int i = 1; i < Q; ++i) { sh += h[i]; sl += l[i]; }
+  // (the low limb balanced: s^2 without its low limb's square is then never negative, as it was
+  // for a small negative s, the sum of populations that cancel)
+  sl += 1 << (kLimb - 1);
   sh += sl >> kLimb;
-  sl &= kMask;
+  sl = (sl & kMask) - (1 << (kLimb - 1));
   // s^2 on the grid that makes b_p s^2 come out on the results', its low limb balanced
   const uint64_t z = shr64((uint64_t)(mul(sh, sh) + (mul(sh, sl) >> (kLimb - 1))), zn);
   const uint64_t zr = z + (1u << (kLimb - 1));
@@ -157,7 +159,7 @@ LBKS_HD bool fix_collide(const uint64_t (&g)[Q], uint64_t (&out)[Q], const FixCo
   LBKS_UNROLL
   for (int p = 0; p < P; ++p) {
     const int64_t th = mul(sh, k.ah[p]);
-    const int64_t tl = mad(sl, k.ah[p], mad(sh, k.al[p], mad(sh >> kHalf, k.ae[p], (1 << (kLimb - 1)) + (k.al[p] >> 1))));
+    const int64_t tl = mad(sl, k.ah[p], mad(sh, k.al[p], mad(sh >> kHalf, k.ae[p], 1 << (kLimb - 1))));
   LBKS_UNROLL
     for (int m = 0; m < 2; ++m) {
       const int i = 2 * p + 1 + m;
