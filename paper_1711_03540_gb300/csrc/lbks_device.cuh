@@ -110,16 +110,20 @@ __device__ __forceinline__ void collide(float (&g)[Q], const Coef<float, Q>& k) 
 // value that is not finite, far out of scale or much smaller than the others) in FP64
 // arithmetic.  Which of the two a site takes depends on its own values alone.
 template <int Q>
-__device__ __forceinline__ void collide(double (&g)[Q], const Coef<double, Q>& k) {
+__device__ __forceinline__ void collide(double (&g)[Q], const FixCoef& fix, const RunDesc* d) {
   uint64_t in[Q], out[Q];
 #pragma unroll
   for (int i = 0; i < Q; ++i) in[i] = (uint64_t)__double_as_longlong(g[i]);
-  if (fix_collide<Q>(in, out, k.fix)) {
+  if (fix.z0 != 0 && fix_collide<Q>(in, out, fix)) {
 #pragma unroll
     for (int i = 0; i < Q; ++i) g[i] = __longlong_as_double((long long)out[i]);
   } else {
-    collide_rn<Q, double>(g, *k.d);
+    collide_rn<Q, double>(g, *d);
   }
+}
+template <int Q>
+__device__ __forceinline__ void collide(double (&g)[Q], const Coef<double, Q>& k) {
+  collide<Q>(g, k.fix, k.d);
 }
 
 __device__ __forceinline__ int64_t wrap_site(int64_t x, int64_t N) {

@@ -116,6 +116,11 @@ __global__ void __launch_bounds__(NTM, MINB)
     for (int i = 0; i < Q; ++i, fs += src.plane) g[i] = *fs;
   }
   const Coef<CT, Q> k = load_coef<CT, Q>(d);
+  __shared__ FixCoef held[(ST == kF64 && !ONE) ? kBlockedPieces : 1];
+  if constexpr (ST == kF64 && !ONE) {
+    if (j == 0) held[q] = d.fix;
+    __syncthreads();
+  }
   CT* const own = &ex[0][0][t + (kGuard ? C * (2 * q + 1) : 0)];
   int from[Q];  // plane i's new value: the column of the thread holding x - c_i, less this one's
 #pragma unroll
@@ -134,7 +139,8 @@ __global__ void __launch_bounds__(NTM, MINB)
     if (s == ksteps - kNextGrid || (s == 0 && ksteps < kNextGrid)) allow_next_grid();
     CT* const xs = own + (s & 1) * (Q - 1) * XS;
     if (active && (!RES || !fixed || s < 3)) {
-      collide<Q>(g, k);
+      if constexpr (ST == kF64) collide<Q>(g, ONE ? k.fix : held[q], &d);
+      else collide<Q>(g, k);
 #pragma unroll
       for (int i = 1; i < Q; ++i) {
         const int c = (i + 1) / 2;

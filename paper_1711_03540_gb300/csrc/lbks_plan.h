@@ -191,10 +191,10 @@ struct BlockedCost {
 };
 inline BlockedCost blocked_cost(int Q, bool f64, bool collapse) {
   BlockedCost c = collapse ? (f64 ? BlockedCost{0.10, 0.21, 3.2, 1, 512} : BlockedCost{0.10, 0.007, 3.2, 4, 512})
-                           : (f64 ? BlockedCost{0.27, 0.095, 1.6, 4, 384} : BlockedCost{0.07, 0.0075, 1.6, 4, 512});
+                           : (f64 ? BlockedCost{0.38, 0.11, 1.6, 4, 384} : BlockedCost{0.07, 0.0075, 1.6, 4, 512});
   if (Q == 5) {
-    c.t0 *= 0.7;
-    c.t1 *= 0.7;
+    c.t0 *= f64 && !collapse ? 0.76 : 0.7;
+    c.t1 *= f64 && !collapse ? 0.76 : 0.7;
   }
   return c;
 }
@@ -484,7 +484,7 @@ struct ClusterTiling {
 // to 1.56 times their rate where clusters were chosen (front tests of 122 lattices: D1Q7
 // 2.86 -> 2.23 us per step, D1Q5 2.01 -> 1.41).
 inline ClusterTiling choose_clusters(const std::vector<int64_t>& Ns, bool reservoir, int Q, int sms, int kwhole) {
-  const double t0 = Q == 7 ? 0.70 : 0.58, t1 = Q == 7 ? 0.08 : 0.058;
+  const double t0 = Q == 7 ? 0.74 : 0.62, t1 = Q == 7 ? 0.085 : 0.064;
   const int C = (Q - 1) / 2;
   const size_t stride = (Ns.size() + 127) / 128;
   std::vector<int64_t> n;
