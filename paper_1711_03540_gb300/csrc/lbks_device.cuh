@@ -106,20 +106,26 @@ __device__ __forceinline__ void collide(float (&g)[Q], const Coef<float, Q>& k) 
   collide_rn<Q, float>(g, k);
 }
 
-// FP64: in fixed point on the integer pipes (fix_collide); a site it does not cover (a
-// value that is not finite, far out of scale or much smaller than the others) in FP64
+// FP64: in fixed point on the integer pipes (fix_collide); a run it is not for (FixCoef::z0 = 0)
+// and a site it does not cover (a value that is not finite or far out of scale) in FP64
 // arithmetic.  Which of the two a site takes depends on its own values alone.
 template <int Q>
 __device__ __forceinline__ void collide(double (&g)[Q], const FixCoef& fix, const RunDesc* d) {
   uint64_t in[Q], out[Q];
 #pragma unroll
   for (int i = 0; i < Q; ++i) in[i] = (uint64_t)__double_as_longlong(g[i]);
-  if (fix.z0 != 0 && fix_collide<Q>(in, out, fix)) {
+  if (fix.z0 != 0) {
+    if (fix_collide<Q>(in, out, fix)) {
 #pragma unroll
-    for (int i = 0; i < Q; ++i) g[i] = __longlong_as_double((long long)out[i]);
-  } else {
-    collide_rn<Q, double>(g, *d);
+      for (int i = 0; i < Q; ++i) g[i] = __longlong_as_double((long long)out[i]);
+      return;
+    }
+    uint64_t any = 0;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) any |= in[i] << 1;
+    if (any == 0) return;  // a site at rest (zeros of either sign) stays as it is
   }
+  collide_rn<Q, double>(g, *d);
 }
 template <int Q>
 __device__ __forceinline__ void collide(double (&g)[Q], const Coef<double, Q>& k) {
