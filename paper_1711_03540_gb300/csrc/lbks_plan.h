@@ -199,39 +199,54 @@ inline BlockedCost blocked_cost(int Q, bool f64, bool collapse) {
   return c;
 }
 
+// Lengths (plus `ghosts`) in decreasing order: all of up to 129, else the longest and 128 of the
+// others, evenly by rank.
+inline std::vector<int64_t> length_sample(const std::vector<int64_t>& Ns, int64_t ghosts) {
+  std::vector<int64_t> n(Ns);
+  for (int64_t& v : n) v += ghosts;
+  std::sort(n.begin(), n.end(), std::greater<int64_t>());
+  if (n.size() > 129) {
+    const size_t others = n.size() - 1;
+    for (size_t q = 0; q < 128; ++q) n[1 + q] = n[1 + (2 * q + 1) * others / 256];
+    n.resize(129);
+  }
+  return n;
+}
+
 // The cheapest tiling.  More steps per launch mean fewer launches and wider halos, which
 // cost warps; smaller blocks spread a small workload over more SMs.  FP64 blocks of more
 // than 128 threads step 8 to 20 % slower on a full device (their warps meet at the barrier
-// and then want the same pipe).  The lattices of a large batch are sampled.
+// and then want the same pipe).  Of a large batch the longest lattice, which decides whether all
+// fit a block, and 128 of the others in order of length (so that the caller's order does not
+// matter) are looked at.
 inline BlockedTiling choose_blocked(const std::vector<int64_t>& Ns, bool reservoir, int Q, const BlockedCost& cost,
                                     int sms, int kwhole) {
   const int C = (Q - 1) / 2;
-  const size_t stride = (Ns.size() + 127) / 128;
+  const std::vector<int64_t> n = length_sample(Ns, reservoir ? 2 * C : 0);
+  const double each = n.size() > 1 ? (double)(Ns.size() - 1) / (double)(n.size() - 1) : 0.0;  // of n[1], n[2], ...
   BlockedTiling best;
   for (int NT : {64, 96, 128, 192, 256, 384, 512}) {
     if (NT > cost.max_threads) break;
     for (int k : {2, 3, 4, 6, 8, 12, 16, 24, 32, 48}) {
       const int64_t h = (int64_t)C * k, room = NT - 2 * h;
       if (room <= 0) break;
-      bool whole = true;
+      const bool whole = n[0] <= NT;
       double pieces = 0.0, small = 0.0;  // stretches and whole lattices; the latter's threads
       int64_t widest = 0;
-      for (size_t r = 0; r < Ns.size(); r += stride) {
-        const int64_t n = Ns[r] + (reservoir ? 2 * C : 0);
-        if (n <= NT) {
-          pieces += 1.0;
-          small += (double)std::max<int64_t>(n, NT / kBlockedPieces) / (0.93 * NT);
-          widest = std::max(widest, n);
+      for (size_t r = 0; r < n.size(); ++r) {
+        const double w = r ? each : 1.0;
+        if (n[r] <= NT) {
+          pieces += w;
+          small += w * (double)std::max<int64_t>(n[r], NT / kBlockedPieces) / (0.93 * NT);
+          widest = std::max(widest, n[r]);
         } else {
-          const int64_t nseg = (n + room - 1) / room;
-          whole = false;
-          pieces += (double)nseg;
-          small += (double)nseg;
-          widest = std::max(widest, (n + nseg - 1) / nseg + 2 * h);
+          const int64_t nseg = (n[r] + room - 1) / room;
+          pieces += w * (double)nseg;
+          small += w * (double)nseg;
+          widest = std::max(widest, (n[r] + nseg - 1) / nseg + 2 * h);
         }
       }
-      pieces *= (double)stride;
-      const double blocks = std::max(1.0, small * (double)stride);
+      const double blocks = std::max(1.0, small);
       BlockedTiling b;
       b.NT = NT;
       b.k = whole ? kwhole : k;
@@ -486,11 +501,8 @@ struct ClusterTiling {
 inline ClusterTiling choose_clusters(const std::vector<int64_t>& Ns, bool reservoir, int Q, int sms, int kwhole) {
   const double t0 = Q == 7 ? 0.74 : 0.62, t1 = Q == 7 ? 0.085 : 0.064;
   const int C = (Q - 1) / 2;
-  const size_t stride = (Ns.size() + 127) / 128;
-  std::vector<int64_t> n;
-  for (size_t r = 0; r < Ns.size(); r += stride) n.push_back(Ns[r] + (reservoir ? 2 * C : 0));
-  std::sort(n.begin(), n.end(), std::greater<int64_t>());
-  const int64_t longest = *std::max_element(Ns.begin(), Ns.end()) + (reservoir ? 2 * C : 0);
+  const std::vector<int64_t> n = length_sample(Ns, reservoir ? 2 * C : 0);
+  const int64_t longest = n.front();
   ClusterTiling best;
   for (int CL : {2, 4, 8})
     for (int NT : {64, 96, 128, 192, 256, 384}) {
@@ -503,7 +515,7 @@ inline ClusterTiling choose_clusters(const std::vector<int64_t>& Ns, bool reserv
         if (b == room.size()) room.push_back(cap);
         room[b] -= std::max(v, pmin) + (v > NT ? pmin : pmin / 2);
       }
-      const double blocks = (double)(room.size() * stride) * CL, per = (double)(768 / NT);
+      const double blocks = (double)room.size() * (double)Ns.size() / (double)n.size() * CL, per = (double)(768 / NT);
       const double even = 0.95 * sms, hold = per * (cap > 1536 ? 0.85 : 0.95) * sms, full = std::floor(blocks / hold);
       const double rest = std::ceil((blocks - full * hold) / even - 1e-9);
       const double slow = cap > 1536 ? 1.15 : NT > 256 ? 1.08 : 1.0;
