@@ -79,7 +79,7 @@ extern "C" {
 
 /* Kernel family. */
 #define LB_KS_KERNEL_AUTO 0     /* resident when every run fits its constraints, else plain (F64) / stream */
-#define LB_KS_KERNEL_PLAIN 1    /* one thread per site, one launch per step (F64, F32); reservoir ends: many steps per launch */
+#define LB_KS_KERNEL_PLAIN 1    /* one thread per site, one launch per step (F64, F32) */
 #define LB_KS_KERNEL_STREAM 2   /* HBM-streaming tiles, one launch per step (F32, F16S) */
 #define LB_KS_KERNEL_RESIDENT 3 /* register-resident, many steps per launch (F64, F32, F16S) */
 /* tau = 1 only (every run): at tau = 1 the BGK collision of Eq. LB_equation_ordinary
@@ -204,11 +204,12 @@ LB_KS_API int lb_ks_batch_init(lb_ks_t **h, int scheme, int32_t nruns, const int
  * f^eq(rho_right[r]) (j >= N[r]-1) every step, so populations streaming in
  * from outside carry the boundary state and those streaming out are dropped.
  * rho0 (sum N[r] values, host or device) initialises the nodes; its two end
- * values are replaced by the boundary values.  These lattices run on the plain
- * kernel family (every node collides once and pushes plane i to node j + c_i when
- * that node is interior), or on the tau = 1 collapse when opts->kernel is
- * LB_KS_KERNEL_COLLAPSE; the guard's
- * re-centring is not allowed (mass flows through the ends: recentre_every must
+ * values are replaced by the boundary values.  Every node collides once and
+ * pushes plane i to node j + c_i when that node is interior: one site per thread and
+ * many steps per launch with opts->kernel AUTO (F64, F32), one step per launch with
+ * PLAIN, with steps_per_launch 1 or another of the tiling options set, and in scaled FP16; the
+ * results are the same bits.  On the tau = 1 collapse when opts->kernel is
+ * LB_KS_KERNEL_COLLAPSE (the tiling options likewise).  The guard's re-centring is not allowed (mass flows through the ends: recentre_every must
  * be 0); lb_ks_rho and lb_ks_mass_energy cover the N[r] nodes.
  * Errors: as lb_ks_batch_init, plus LB_KS_EINVAL for NULL or non-finite
  * boundary values, opts->kernel STREAM/RESIDENT, or recentre_every != 0.
@@ -276,7 +277,9 @@ LB_KS_API int64_t lb_ks_steps_done(const lb_ks_t *h);
  * sites per thread (1: the one-site-per-thread resident kernel, the automatic choice for
  * F64 and for F32 batches too small to fill the device), threads per block, steps per launch
  * and blocks per work group of whole lattices (1 or 2, with one site per thread up to 8; all 0
- * when not resident), number of runs and total sites.  Any pointer may be NULL.
+ * when not resident), number of runs and total sites.  Lattices with fixed-value ends
+ * report LB_KS_KERNEL_PLAIN, or COLLAPSE, and the others as for one site per thread where they
+ * run many steps per launch.  Any pointer may be NULL.
  */
 LB_KS_API int lb_ks_describe(const lb_ks_t *h, int *kernel, int *sites_per_thread, int *threads_per_block,
                    int *steps_per_launch, int *cluster_size, int32_t *nruns, int64_t *total_sites);
@@ -295,7 +298,7 @@ LB_KS_API int lb_ks_describe(const lb_ks_t *h, int *kernel, int *sites_per_threa
  *       (0: none are)
  *   [6] 1 if single-block bundles run two to a pair work group on this lane's queue
  *   [7] lattices held as two halves
- * Returns the number of lanes (0 when the handle does not run the resident kernels),
+ * Returns the number of lanes (0 when the handle runs one step per launch),
  * or LB_KS_EINVAL (h NULL, max_lanes < 0, lanes NULL with max_lanes > 0).
  */
 #define LB_KS_LANE_FIELDS 8

@@ -1096,14 +1096,18 @@ int create_body(lb_ks*& h, lb_ks_t** out, int scheme, int32_t nruns, const int64
       rc = setup_resident(h, false);
       if (rc < 0) return bail(rc);
       h->collapse_resident = rc == 0;
-    } else if (reservoir && o.steps_per_launch != 1) {
+    } else if (reservoir && free_tiling(h)) {
       int sms = 0;
       if ((rc = sm_count(h, &sms)) || (rc = setup_blocked(h, sms, 1e300)) < 0) return bail(rc);
     }
   } else if (reservoir) {
-    kern = LB_KS_KERNEL_PLAIN;
+    // many steps per launch, unless one (kernel PLAIN, steps_per_launch 1) or a tiling that the
+    // one-site-per-thread kernel does not have is asked for
     int sms = 0;
-    if ((rc = sm_count(h, &sms)) || (h->prec != kF16S && (rc = setup_blocked(h, sms, 1e300)) < 0)) return bail(rc);
+    if (kern == LB_KS_KERNEL_AUTO && h->prec != kF16S && free_tiling(h) &&
+        ((rc = sm_count(h, &sms)) || (rc = setup_blocked(h, sms, 1e300)) < 0))
+      return bail(rc);
+    kern = LB_KS_KERNEL_PLAIN;
   } else if (kern == LB_KS_KERNEL_AUTO || kern == LB_KS_KERNEL_RESIDENT) {
     rc = setup_resident(h, kern == LB_KS_KERNEL_RESIDENT);
     if (rc < 0) return bail(rc);
@@ -1442,7 +1446,7 @@ int lb_ks_set_link_test(lb_ks_t* h, int32_t withhold_step, uint32_t wait_rounds)
 int lb_ks_describe(const lb_ks_t* h, int* kernel, int* spt, int* tpb, int* spl, int* cl, int32_t* nruns,
                    int64_t* total) {
   if (!h) return LB_KS_EINVAL;
-  const bool res = h->kernel == LB_KS_KERNEL_RESIDENT || h->collapse_resident;
+  const bool res = h->nlanes > 0;
   if (kernel) *kernel = h->kernel;
   if (spt) *spt = res ? h->S : 0;
   if (tpb) *tpb = res ? h->NT : 0;
@@ -1458,7 +1462,6 @@ int lb_ks_describe(const lb_ks_t* h, int* kernel, int* spt, int* tpb, int* spl, 
 
 int lb_ks_describe_lanes(const lb_ks_t* h, int32_t* lanes, int max_lanes) {
   if (!h || max_lanes < 0 || (max_lanes > 0 && !lanes)) return LB_KS_EINVAL;
-  if (!(h->kernel == LB_KS_KERNEL_RESIDENT || h->collapse_resident)) return 0;
   for (int l = 0; l < h->nlanes && l < max_lanes; ++l) {
     const Lane& L = h->lanes[l];
     int32_t* r = lanes + LB_KS_LANE_FIELDS * l;
