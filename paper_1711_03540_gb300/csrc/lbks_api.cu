@@ -720,10 +720,26 @@ bool has_pair_lattices(const lb_ks* h, int S, int NT) {
   return false;
 }
 
+// f = f^eq(rho0) in the first arena (the tau = 1 collapse: rho0 - rhobar in both, as fixed ends
+// and ghosts keep their values in both), on the handle's stream.
+int init_populations(lb_ks* h) {
+  if (h->kernel == LB_KS_KERNEL_COLLAPSE) {
+    for (int b = 0; b < 2; ++b)
+      LBKS_CUDA(h, launch_collapse_init(h->prec, arena(h, b), h->d_runs, h->d_plain_tiles, h->n_plain_tiles, h->d_stage,
+                                        h->d_rho_off, h->stream), "init");
+    h->launches += 2;
+    return LB_KS_OK;
+  }
+  LBKS_CUDA(h, launch_init_eq(h->Q, h->prec, arena(h, 0), h->d_runs, h->d_stream_tiles, h->n_stream_tiles, h->d_stage,
+                              h->d_rho_off, h->stream), "init");
+  h->launches += 1;
+  return LB_KS_OK;
+}
+
 // Autotuner of the resident kernel: times a few tilings (sites per thread, threads per
 // block), ring work-group sizes (one block or a cluster pair) and lane splits on this
-// handle's own lattices for a short run, and keeps the fastest.  Runs before the state
-// is initialised, on the zeroed arenas (the kernel's work does not depend on the values).
+// handle's own lattices for a short run from its own initial state (the FP64 collision's
+// work depends on the values: a site at rest does next to nothing), and keeps the fastest.
 int autotune_resident(lb_ks* h) {
   struct Cand { int S, NT; double w; int cl; int merge; int kx; };
   std::vector<Cand> cands;
@@ -769,6 +785,9 @@ int autotune_resident(lb_ks* h) {
     if (h->nlanes < 2 && c.w != 1.0) continue;  // the split weight only matters with more than one lane
     int64_t nk = 0;
     for (int rep = 0; rep < 2 && rc == LB_KS_OK; ++rep) {  // first repetition warms up
+      h->cur = 0;
+      h->phase = 0;
+      if ((rc = init_populations(h)) != LB_KS_OK) break;
       cudaEventRecord(e0, h->stream);
       rc = issue_steps(h, trial, h->stream, &nk);
       cudaEventRecord(e1, h->stream);
@@ -791,11 +810,14 @@ int autotune_resident(lb_ks* h) {
   } else if ((rc = setup_resident(h, true)) != LB_KS_OK) {
     return rc;
   }
-  // the trials advanced the (zero) state: start the real run from the first arena
+  // the trials advanced the state: the real run starts from cleared arenas, in the first one
   h->cur = 0;
   h->steps_done = 0;
   h->phase = 0;
   h->launches = 0;
+  for (void* f : h->fbuf)
+    LBKS_CUDA(h, cudaMemsetAsync(f, 0, storage_bytes(h->prec) * (size_t)h->nplanes * (size_t)h->plane, h->stream),
+              "clear populations");
   LBKS_CUDA(h, cudaMemsetAsync(h->d_flags, 0, sizeof(int), h->stream), "clear flags");
   return LB_KS_OK;
 }
@@ -1116,6 +1138,8 @@ int create_body(lb_ks*& h, lb_ks_t** out, int scheme, int32_t nruns, const int64
   h->kernel = kern;
   if (kern == LB_KS_KERNEL_STREAM && (ce = stream_prepare(scheme, h->prec)) != cudaSuccess)
     return bail(cuda_fail(h, ce, "stream kernel setup"));
+  if ((kern == LB_KS_KERNEL_COLLAPSE || kern == LB_KS_KERNEL_PLAIN || reservoir) && (rc = plain_tiles()) != LB_KS_OK)
+    return bail(rc);
   // streams and events for concurrent lanes, when the plan has several (or the tuner
   // may choose one that does)
   if ((kern == LB_KS_KERNEL_RESIDENT || h->collapse_resident) && (o.autotune || h->nlanes > 1)) {
@@ -1129,29 +1153,14 @@ int create_body(lb_ks*& h, lb_ks_t** out, int scheme, int32_t nruns, const int64
   }
   if (h->nlanes > 1 && !h->ev_fork) return bail(fail(h, LB_KS_ECUDA, "internal: lanes without their streams"));
 
-  if ((kern == LB_KS_KERNEL_COLLAPSE || kern == LB_KS_KERNEL_PLAIN || reservoir) && (rc = plain_tiles()) != LB_KS_OK)
-    return bail(rc);
   if ((ce = join_init()) != cudaSuccess) return bail(cuda_fail(h, ce, "join init"));
-  if (kern == LB_KS_KERNEL_COLLAPSE) {
-    // rho - rhobar in both arenas (reservoir ends and ghosts keep their values in both)
+  if ((rc = init_populations(h)) != LB_KS_OK) return bail(rc);
+  if (reservoir && kern != LB_KS_KERNEL_COLLAPSE) {  // end nodes and ghosts at f^eq(rho_bc)
     for (int b = 0; b < 2; ++b)
-      if ((ce = launch_collapse_init(h->prec, arena(h, b), h->d_runs, h->d_plain_tiles, h->n_plain_tiles, h->d_stage,
-                                     h->d_rho_off, h->stream)) != cudaSuccess)
-        return bail(cuda_fail(h, ce, "init"));
+      if ((ce = launch_reservoir_step(scheme, h->prec, arena(h, b), arena(h, b), h->d_runs, h->d_plain_tiles,
+                                      h->n_plain_tiles, h->plain_tile, 1, h->stream)) != cudaSuccess)
+        return bail(cuda_fail(h, ce, "reservoir init"));
     h->launches += 2;
-  } else {
-    // f = f^eq(rho0)
-    if ((ce = launch_init_eq(scheme, h->prec, arena(h, 0), h->d_runs, h->d_stream_tiles, h->n_stream_tiles, h->d_stage,
-                             h->d_rho_off, h->stream)) != cudaSuccess)
-      return bail(cuda_fail(h, ce, "init"));
-    h->launches += 1;
-    if (reservoir) {  // end nodes and ghosts at f^eq(rho_bc)
-      for (int b = 0; b < 2; ++b)
-        if ((ce = launch_reservoir_step(scheme, h->prec, arena(h, b), arena(h, b), h->d_runs, h->d_plain_tiles,
-                                        h->n_plain_tiles, h->plain_tile, 1, h->stream)) != cudaSuccess)
-          return bail(cuda_fail(h, ce, "reservoir init"));
-      h->launches += 2;
-    }
   }
   if ((ce = cudaStreamSynchronize(h->stream)) != cudaSuccess) return bail(cuda_fail(h, ce, "init sync"));
   // rho0's statistics, computed on the device while the host planned
