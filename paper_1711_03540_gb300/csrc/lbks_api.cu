@@ -468,7 +468,7 @@ int setup_resident(lb_ks* h, bool required, int S_force = 0, int NT_force = 0, d
     const int kring = h->opts.steps_per_launch ? h->opts.steps_per_launch : (R > 0 ? std::min(R, 1000) : 1000);
     int kseg = h->opts.steps_per_launch ? h->opts.steps_per_launch
                : chosen && fixed.kseg    ? fixed.kseg
-                                        : std::max(1, (int)((int64_t)NT * S / (20 * h->cmax)));
+                                        : segment_steps(S, NT, h->cmax);
     kseg = std::min(kseg, kring);
     // default: cluster pairs when some lattice needs more than one block and fits two
     int cl = cl_force ? cl_force : h->opts.cluster_size;
@@ -756,8 +756,10 @@ int autotune_resident(lb_ks* h) {
   } else {
     tilings = {{20, 256}, {18, 256}, {12, 384}, {16, 256}, {8, 512}};
   }
+  int kseg = 1;
   for (auto& tl : tilings) {
     const int NT = tl.second ? tl.second : (col ? 256 : default_threads(h->prec, tl.first));
+    kseg = std::max(kseg, segment_steps(tl.first, NT, h->cmax));
     for (int cl : {2, 1}) {
       if (col && cl == 2) continue;
       if (h->opts.cluster_size && cl != h->opts.cluster_size) continue;
@@ -770,9 +772,9 @@ int autotune_resident(lb_ks* h) {
     }
   }
   if (cands.empty()) return LB_KS_OK;  // keep the plan made before tuning
-  // one full whole-lattice launch per trial (500 steps, or fewer when the guard
-  // interval or steps_per_launch is shorter), so the launch edges weigh as in a run
-  const int64_t trial = std::max<int64_t>(2 * h->kseg, std::min<int64_t>(h->kmax, 500));
+  const int R = h->opts.recentre_every;
+  const int kring = h->opts.steps_per_launch ? h->opts.steps_per_launch : (R > 0 ? std::min(R, 1000) : 1000);
+  const int64_t trial = tuner_steps(kring, std::min(kseg, kring));
   cudaEvent_t e0, e1;
   LBKS_CUDA(h, cudaEventCreate(&e0), "tuner event");
   LBKS_CUDA(h, cudaEventCreate(&e1), "tuner event");

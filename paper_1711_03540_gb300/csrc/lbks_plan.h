@@ -129,6 +129,14 @@ inline bool plan_pieces(const std::vector<int64_t>& Ns, int C, int S, int NT, in
   return true;
 }
 
+// Steps per launch of the fixed rule for segments of NT S sites: halos of a tenth on each side.
+inline int segment_steps(int S, int NT, int C) { return std::max(1, (int)((int64_t)NT * S / (20 * C))); }
+
+// Steps of every trial of the autotuner, whatever tiling a trial runs: one launch of whole
+// lattices (kring steps, at most 500), so that launch edges weigh as in a run, and two at least
+// of the longest segments (kseg steps) among the trials.
+inline int64_t tuner_steps(int kring, int kseg) { return std::max<int64_t>(2LL * kseg, std::min(kring, 500)); }
+
 // Pieces a block of the one-site-per-thread kernel holds at most (plan_blocked gives each
 // at least its share of the block's threads).
 constexpr int kBlockedPieces = 16;
