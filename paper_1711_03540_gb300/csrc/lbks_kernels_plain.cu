@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(kPlainThreads) gather_rho_kernel(Arena src, co
 // The plain fused step: one thread per site reads its Q populations, collides
 // (Eq. LB_equation_ordinary) and pushes f*_i to site x + c_i (mod N).
 template <int Q, int ST>
-__global__ void __launch_bounds__(kPlainThreads) plain_step_kernel(Arena src, Arena dst,
+__global__ void __launch_bounds__(kPlainThreads, ST == kF64 ? 3 : 1) plain_step_kernel(Arena src, Arena dst,
                                                                    const RunDesc* __restrict__ runs,
                                                                    const Tile* __restrict__ tiles) {
   using T = typename StorageType<ST>::type;
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(kPlainThreads) plain_step_kernel(Arena src, Ar
 // pushes plane i to j + c_i when that node is interior (pushes into reservoir
 // nodes are dropped), so each interior node receives exactly one value per plane.
 template <int Q, int ST>
-__global__ void __launch_bounds__(kPlainThreads) reservoir_step_kernel(Arena src, Arena dst,
+__global__ void __launch_bounds__(kPlainThreads, ST == kF64 ? 3 : 1) reservoir_step_kernel(Arena src, Arena dst,
                                                                        const RunDesc* __restrict__ runs,
                                                                        const Tile* __restrict__ tiles, int reset_only) {
   using T = typename StorageType<ST>::type;
