@@ -1088,6 +1088,9 @@ int create_body(lb_ks*& h, lb_ks_t** out, int scheme, int32_t nruns, const int64
       (ce = up(h->d_rho_off, h->rho_off.data(), sizeof(int64_t) * h->rho_off.size())) != cudaSuccess ||
       (ce = cudaMemset(h->d_flags, 0, sizeof(int))) != cudaSuccess)
     return bail(cuda_fail(h, ce, "upload"));
+  // (copies from pageable memory may return before they have reached the device; the capture
+  // stream does not wait for the default stream's work)
+  if ((ce = cudaStreamSynchronize(cudaStreamLegacy)) != cudaSuccess) return bail(cuda_fail(h, ce, "upload"));
   for (int b = 0; b < 2; ++b)
     if ((ce = cudaMemsetAsync(h->fbuf[b], 0, fbytes, is)) != cudaSuccess)
       return bail(cuda_fail(h, ce, "clear populations"));
@@ -1416,6 +1419,9 @@ int lb_ks_load(lb_ks_t* h, const void* buf, size_t bytes) try {
   h->mass0_h = m0;
   h->tables_on_host = true;
   LBKS_CUDA(h, cudaMemcpy(h->d_runs, runs.data(), sizeof(RunDesc) * h->nruns, cudaMemcpyHostToDevice), "load runs");
+  // (a copy from pageable memory may return before it has reached the device, and the handle's
+  // stream need not wait for the default stream's work)
+  LBKS_CUDA(h, cudaStreamSynchronize(cudaStreamLegacy), "load runs");
   if (h->zb && !zero_terms(h)) {
     // the loaded constants have such a term: the general kernels from now on
     h->zb = false;
@@ -1437,6 +1443,7 @@ int lb_ks_load(lb_ks_t* h, const void* buf, size_t bytes) try {
   h->phase = R > 0 ? hdr2[2] % R : 0;
   h->sticky = LB_KS_OK;
   LBKS_CUDA(h, cudaMemset(h->d_flags, 0, sizeof(int)), "clear flags");
+  LBKS_CUDA(h, cudaStreamSynchronize(cudaStreamLegacy), "load");
   return LB_KS_OK;
 } catch (...) {
   return abi_exception(h);
