@@ -340,13 +340,23 @@ cudaError_t prepared(int kind, int Q, int prec, int S, int NT, bool zb, int* out
   return cudaSuccess;
 }
 
+void release_lanes(lb_ks* h);
+
 // Plan of the blocked kernel (one site per thread), lattices over the blocks of a cluster or in
-// haloed stretches, if its step is estimated to take less than `than` microseconds: LB_KS_OK, 1 if not, or an error.
+// haloed stretches, if its step is estimated to take less than `than` microseconds: LB_KS_OK, 1
+// if not, or an error.  1 also where its piece tables (40 bytes per 116 sites of a long lattice,
+// ten times the register-resident kernel's) do not fit beside the arenas.
 int setup_blocked(lb_ks* h, int sms, double than) {
   const int R = h->opts.recentre_every;
   const int kwhole = R > 0 ? std::min(R, 1000) : 1000;
   const BlockedCost cost = blocked_cost(h->Q, h->prec == kF64, h->nplanes == 1);
   const BlockedTiling b = choose_blocked(h->N, h->reservoir, h->Q, cost, sms, kwhole);
+  const auto no_room = [h](int rc) {
+    if (rc != LB_KS_ENOMEM) return rc;
+    release_lanes(h);
+    h->err = "no error";
+    return 1;
+  };
   std::vector<Piece> pieces;
   if (h->prec == kF64 && h->nplanes > 1) {
     const ClusterTiling c = choose_clusters(h->N, h->reservoir, h->Q, sms, kwhole);
@@ -354,7 +364,7 @@ int setup_blocked(lb_ks* h, int sms, double than) {
     if (c.us < 0.92 * std::min(b.us, than) && plan_clusters(h->N, h->reservoir, h->cmax, c.NT, c.CL, &pieces, &bundles)) {
       Lane& L = h->lanes[0];
       int rc;
-      if ((rc = upload_lane(h, &L, pieces, bundles, c.CL, kwhole, false, 1.0))) return rc;
+      if ((rc = upload_lane(h, &L, pieces, bundles, c.CL, kwhole, false, 1.0))) return no_room(rc);
       L.grid = L.nbundles / c.CL;
       L.one = L.spread = false;
       h->nlanes = 1;
@@ -374,7 +384,7 @@ int setup_blocked(lb_ks* h, int sms, double than) {
   blocked_bundles(pieces, b.NT, b.spread, &bundles);
   Lane& L = h->lanes[0];
   int rc;
-  if ((rc = upload_lane(h, &L, pieces, bundles, 1, b.k, segmented, 1.0))) return rc;
+  if ((rc = upload_lane(h, &L, pieces, bundles, 1, b.k, segmented, 1.0))) return no_room(rc);
   if (bundles.empty()) L.nbundles = (int)pieces.size();
   L.grid = L.nbundles;
   L.one = bundles.empty();
