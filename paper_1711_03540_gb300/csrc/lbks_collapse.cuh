@@ -46,7 +46,10 @@ __device__ __forceinline__ CollapseCoef<CT, C> load_collapse_coef(const RunDesc&
 // the collapse family calls this with the same operands, so their results agree
 // bitwise.
 // ZB: B_3 is zero (D1Q7's default weights), so that its term, four of the 22 operations, is
-// an addition of zero.  ZR: rhobar is zero (FP64 storage), and so is what is added to s.
+// an addition of zero (while the squares are finite: once one overflows, its term is
+// 0 x infinity three sites away, where a NaN would come; the neighbours one and two away are infinite
+// in both, and the guard's mass is not finite at the same step).  ZR: rhobar is zero (FP64
+// storage), and so is what is added to s.
 template <typename CT, int C, bool ZB = false, bool ZR = false>
 __device__ __forceinline__ CT collapse_site(CT d0, const CT (&dl)[C + 1], const CT (&dr)[C + 1],
                                             const CollapseCoef<CT, C>& k) {

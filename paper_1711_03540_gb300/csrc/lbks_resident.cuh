@@ -217,7 +217,9 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* m, uint32_t parity) {
 // Post-collision value of one plane (post_collision in lbks_device.cuh).  NOB: the plane's
 // b is zero, so that rho^2 b + t is t: the c = +-3 planes of D1Q7, whose first-moment
 // weights w1 are zero (Sec. 2.3; not with the full-inverse weights), saving 2 of a site's 29
-// FP32 instructions.
+// FP32 instructions.  The same bits as with the term while rho^2 is finite.  Once it overflows,
+// the term is 0 x infinity there and these two planes NaN, finite here; the site's others are infinite and its
+// g_0 NaN in both, so that the guard's mass is not finite at the same step.
 template <bool NOB, typename CT>
 __device__ __forceinline__ CT post_plane(CT r, CT g, CT rho2, CT b, CT t) {
   if constexpr (NOB) return fma_rn(r, g, t);
