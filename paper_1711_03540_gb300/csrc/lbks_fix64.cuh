@@ -210,9 +210,10 @@ LBKS_HD bool fix_collide(const uint64_t (&g)[Q], uint64_t (&out)[Q], const FixCo
   // results in units of half the planes' grids: even + odd and even - odd
   const int32_t rhalf = k.rl >> 1;
   int64_t y[Q];
+  uint32_t low = 0xffffffffu;
   uint64_t f = 0;  // what y0 holds below its unit, in 2^-32 of it
   LBKS_UNROLL
-  for (int p = 0; p < P; ++p) {
+  for (int p = P - 1; p >= 0; --p) {
     const int i = 2 * p + 1, j = i + 1;
     const int64_t el = mad(l[i], k.rh, mad(h[i], k.rl, mad(sg[i], rhalf, 1 << (kLimb - 1))));
     const int64_t ol = mad(l[j], k.rh, mad(h[j], k.rl, mad(sg[j], rhalf, 1 << (kLimb - 1))));
@@ -221,18 +222,23 @@ LBKS_HD bool fix_collide(const uint64_t (&g)[Q], uint64_t (&out)[Q], const FixCo
     y[i] = even + odd;
     y[j] = even - odd;
     const int64_t d = mad(h[i], 1 << kLimb, (int64_t)l[i]) - even;
+    if (p == 2) {
+      out[i] = to_fp64(y[i], (e - (uint32_t)k.kp[p] - 1079u) << 20, low);
+      out[j] = to_fp64(y[j], (e - (uint32_t)k.kp[p] - 1079u) << 20, low);
+    }
     y0 += sra64(d, (uint32_t)k.kp[p]);
     f += below64(d, (uint32_t)k.kp[p]);
   }
   y0 += (int64_t)(f >> 32);
   // g_0 keeps the bits it had room for; what is left goes to the planes +-1, half each (the odd
   // unit to either in turn), but for a sixteenth that the planes +-2 take (so that none takes as
-  // much as a quarter of g_0's last bit; they can where their grid is fine enough).  They take half where the
-  // planes are so small that short waves stay long: four directions make less noise there than two.
+  // much as a quarter of g_0's last bit; where their grid is fine enough).  They take half where
+  // the planes are so small that short waves stay long: four directions make less noise than two.
   const uint32_t gap = e - (m0 >> 20), bit = gap < 3u ? 8u >> gap : 1u;
   const int64_t v0 = (y0 + (int64_t)(gap < 3u ? bit >> 1 : (uint32_t)f >> 31)) & -(int64_t)bit;
   const int32_t left = (int32_t)((uint32_t)y0 - (uint32_t)v0);
-  const int32_t far = k.kp[1] < 2 ? 0 : k.kp[0] > 14 ? 2 * left + 1 : (left + 2) >> 2;
+  const int32_t share = k.kp[1] < 2 ? 0 : k.kp[0] > 14 ? 8 : 1;
+  const int32_t far = (left * share + (share < 2 ? 2 * share : 4)) >> 2;
   const uint32_t lo = (uint32_t)f - ((uint32_t)far << 30);
   const int32_t hi = left - (far >> 2) - (lo > (uint32_t)f ? 1 : 0);
   const int32_t near = shl_pair(hi, lo, (uint32_t)k.kp[0] + 1u) | (shl32(lo, (uint32_t)k.kp[0] + 1u) ? 1 : 0);
@@ -241,10 +247,9 @@ LBKS_HD bool fix_collide(const uint64_t (&g)[Q], uint64_t (&out)[Q], const FixCo
   y[2] += near - half;
   y[3] += half2;
   y[4] += half2;
-  uint32_t low = 0xffffffffu;
   out[0] = to_fp64(v0, (e - 1078u) << 20, low);
   LBKS_UNROLL
-  for (int i = 1; i < Q; ++i) out[i] = to_fp64(y[i], (e - (uint32_t)k.kp[(i - 1) / 2] - 1079u) << 20, low);
+  for (int i = 1; i < 5; ++i) out[i] = to_fp64(y[i], (e - (uint32_t)k.kp[(i - 1) / 2] - 1079u) << 20, low);
   if (low == 0u) {  // a result of zero
   LBKS_UNROLL
     for (int i = 0; i < Q; ++i)
