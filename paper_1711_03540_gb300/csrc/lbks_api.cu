@@ -1091,16 +1091,20 @@ int create_body(lb_ks*& h, lb_ks_t** out, int scheme, int32_t nruns, const int64
   if ((rc = dalloc(h, &h->d_delta, nruns))) return bail(rc);
   if ((rc = dalloc(h, &h->d_flags, 1))) return bail(rc);
   if ((rc = dalloc(h, &h->d_bad_run, 1))) return bail(rc);
-  auto up = [&](void* dst, const void* src, size_t bytes) { return cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice); };
+  // (on the stream of the kernels that read them first: a copy from pageable memory may return
+  // before it has reached the device, and that stream does not wait for the default stream's work)
+  CopyWait tables;
+  auto up = [&](void* dst, const void* src, size_t bytes) {
+    return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, is);
+  };
   if ((ce = up(h->d_runs, h->runs_h.data(), sizeof(RunDesc) * nruns)) != cudaSuccess ||
       (ce = up(h->d_stream_tiles, st.data(), sizeof(Tile) * st.size())) != cudaSuccess ||
       (ce = up(h->d_stream_tile_begin, st_begin.data(), sizeof(int32_t) * st_begin.size())) != cudaSuccess ||
       (ce = up(h->d_rho_off, h->rho_off.data(), sizeof(int64_t) * h->rho_off.size())) != cudaSuccess ||
-      (ce = cudaMemset(h->d_flags, 0, sizeof(int))) != cudaSuccess)
+      (ce = cudaMemsetAsync(h->d_flags, 0, sizeof(int), is)) != cudaSuccess ||
+      (ce = cudaEventCreateWithFlags(&tables.ev, cudaEventDisableTiming)) != cudaSuccess ||
+      (ce = cudaEventRecord(tables.ev, is)) != cudaSuccess)
     return bail(cuda_fail(h, ce, "upload"));
-  // (copies from pageable memory may return before they have reached the device; the capture
-  // stream does not wait for the default stream's work)
-  if ((ce = cudaStreamSynchronize(cudaStreamLegacy)) != cudaSuccess) return bail(cuda_fail(h, ce, "upload"));
   for (int b = 0; b < 2; ++b)
     if ((ce = cudaMemsetAsync(h->fbuf[b], 0, fbytes, is)) != cudaSuccess)
       return bail(cuda_fail(h, ce, "clear populations"));

@@ -2,8 +2,10 @@
 should be used: what it guards against is a race).  Tables are copied from pageable memory with
 cudaMemcpy, on the default stream, which may return before the copy has reached the device; the
 handle's and the capture stream need not wait for the default stream.  So a kernel on one of them
-that reads such a table comes after a synchronisation of the default stream."""
+that reads such a table comes after a synchronisation of the default stream, or the copy goes on
+the kernel's stream."""
 import os
+import re
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 WAIT = "cudaStreamSynchronize(cudaStreamLegacy)"
@@ -28,6 +30,10 @@ def test_checkpoint_load():
 
 
 def test_creation():
+    """Here the copies go on the stream of the kernel that reads the tables."""
     body = _function("int create_body(")
-    copy, kernel = body.index("up(h->d_rho_off"), body.index("launch_init_stats(")
-    assert WAIT in body[copy:kernel]
+    up = body[body.index("auto up = "):]
+    assert re.match(r"auto up = \[&\][^{]*\{\s*return cudaMemcpyAsync\([^;]*, is\);", up)
+    kernel = body[body.index("launch_init_stats("):]
+    assert re.match(r"launch_init_stats\([^;]*?,\s*is\)\)", kernel)
+    assert body.index("CopyWait tables;") > body.index("std::vector<Tile> st;")  # (waits before they go)
