@@ -163,7 +163,7 @@ LBKS_HD bool fix_collide(const uint64_t (&g)[Q], uint64_t (&out)[Q], const FixCo
   constexpr int P = (Q - 1) / 2;
   // the site's scale 2^(e - 1022): g_0 below it and the planes +-p kp[p] binades further down
   const uint32_t m0 = hi32(g[0]) & 0x7fffffffu;
-  uint32_t top = m0, least = m0;
+  uint32_t top = m0, least = 0xffffffffu;
   LBKS_UNROLL
   for (int p = 0; p < P; ++p) {
     const uint32_t u = hi32(g[2 * p + 1]) & 0x7fffffffu, v = hi32(g[2 * p + 2]) & 0x7fffffffu;
@@ -174,12 +174,14 @@ LBKS_HD bool fix_collide(const uint64_t (&g)[Q], uint64_t (&out)[Q], const FixCo
   const uint32_t e = top >> 20;
   const uint32_t zn = (uint32_t)k.z0 - e;  // shift of s^2; negative for z0 = 0 (and NaN, infinities)
   int32_t h[Q], l[Q], sg[Q];
-  to_limbs<false>(g[0], e, h[0], l[0], sg[0]);
+  // (g_0 may be far below the scale, about a zero of the density, where the planes are not: a
+  // lattice odd in x has such sites at all times)
+  to_limbs<true>(g[0], e, h[0], l[0], sg[0]);
   LBKS_UNROLL
   for (int i = 1; i < Q; ++i) to_limbs<false>(g[i], e - (uint32_t)k.kp[(i - 1) / 2], h[i], l[i], sg[i]);
   if (e - (least >> 20) > 35u) {
   LBKS_UNROLL
-    for (int i = 0; i < Q; ++i) to_limbs<true>(g[i], e - (i ? (uint32_t)k.kp[(i - 1) / 2] : 0u), h[i], l[i], sg[i]);
+    for (int i = 1; i < Q; ++i) to_limbs<true>(g[i], e - (uint32_t)k.kp[(i - 1) / 2], h[i], l[i], sg[i]);
   }
   // of each pair its sum (in h, l, sg of the first) and difference (of the second); s = sum g_i,
   // rounded to g_0's grid
