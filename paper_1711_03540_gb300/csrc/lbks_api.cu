@@ -361,7 +361,7 @@ int setup_blocked(lb_ks* h, int sms, double than) {
   if (h->prec == kF64 && h->nplanes > 1) {
     const ClusterTiling c = choose_clusters(h->N, h->reservoir, h->Q, sms, kwhole);
     std::vector<int2> bundles;
-    if (c.us < 0.92 * std::min(b.us, than) && plan_clusters(h->N, h->reservoir, h->cmax, c.NT, c.CL, &pieces, &bundles)) {
+    if (c.us < 0.96 * std::min(b.us, than) && plan_clusters(h->N, h->reservoir, h->cmax, c.NT, c.CL, &pieces, &bundles)) {
       Lane& L = h->lanes[0];
       int rc;
       if ((rc = upload_lane(h, &L, pieces, bundles, c.CL, kwhole, false, 1.0))) return no_room(rc);

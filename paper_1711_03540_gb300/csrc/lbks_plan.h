@@ -188,7 +188,7 @@ struct BlockedTiling {
 // 256 to 2^20 sites and of the 4096-lattice ensembles:
 //   t0 + t1 max(w, wmin) + launch / k,
 // w the warps an SM has to step, t1 the issue time of one, wmin one per scheduler (t0 + 4 t1
-// is then the latency of a step: D1Q7 FP64 0.65 us, FP32 0.10 us; the FP64 collapse, in
+// is then the latency of a step: D1Q7 FP64 0.82 us, FP32 0.10 us; the FP64 collapse, in
 // FP64 arithmetic, is bound by the FP64 pipe the schedulers share), launch the time
 // between two launches' work (with several FP64 blocks an SM kMoreLaunch times as long: the
 // last blocks of one launch end apart).
@@ -199,10 +199,10 @@ struct BlockedCost {
 };
 inline BlockedCost blocked_cost(int Q, bool f64, bool collapse) {
   BlockedCost c = collapse ? (f64 ? BlockedCost{0.10, 0.21, 3.2, 1, 512} : BlockedCost{0.10, 0.007, 3.2, 4, 512})
-                           : (f64 ? BlockedCost{0.38, 0.11, 1.6, 4, 384} : BlockedCost{0.07, 0.0075, 1.6, 4, 512});
+                           : (f64 ? BlockedCost{0.48, 0.086, 1.6, 4, 384} : BlockedCost{0.07, 0.0075, 1.6, 4, 512});
   if (Q == 5) {
-    c.t0 *= f64 && !collapse ? 0.76 : 0.7;
-    c.t1 *= f64 && !collapse ? 0.76 : 0.7;
+    c.t0 *= f64 && !collapse ? 0.78 : 0.7;
+    c.t1 *= f64 && !collapse ? 0.78 : 0.7;
   }
   return c;
 }
@@ -506,17 +506,19 @@ struct ClusterTiling {
 };
 
 // The cheapest cluster tiling for FP64 batches with lattices too long for a block.  No halos and
-// no launch ends, but a cluster barrier per step: measured (GB300, D1Q7, 128-thread blocks) 1.02,
-// 1.30, 1.53, 1.84, 2.20, 2.55 us per step with 1 to 6 blocks an SM, t0 + t1 w for w warps.
-// Clusters fill the SMs a little unevenly (144 blocks put two on some of 152 SMs), and blocks
-// beyond 768 threads an SM run all their steps after the others.  Large clusters wait for
-// room for all their blocks (8 x 384: up to 1.7 times the model, not considered; 8 x 256: 1.05
-// to 1.2, and no more than 0.85 of the device at once).  The caller asks for 8 % less than the
-// launches' estimate: over 200 batches of 4 to 1400 lattices of 200 to 2900 sites it gave 1.02
-// to 1.56 times their rate where clusters were chosen (front tests of 122 lattices: D1Q7
-// 2.86 -> 2.23 us per step, D1Q5 2.01 -> 1.41).
+// no launch ends, but a cluster barrier per step: measured (GB300, D1Q7, 4 x 128 clusters that
+// fill the device) 1.13, 1.46, 1.67, 2.16, 3.10 us per step with 1, 2, 3, 4 and 6 blocks an SM,
+// t0 + t1 w for w warps.  A cluster's blocks lie in one GPC, of 18 or 20 SMs, so fewer clusters
+// than SMs / CL have a block an SM each: of eight blocks 16 (17 step as slowly as 36 do, with two
+// blocks on some SMs: 1.44 against 1.45 us), with two blocks an SM 36, with three 52.  Blocks
+// beyond 768 threads an SM run all their steps after the others.  Blocks of 256 threads take 1.09
+// times that, others but 128 1.1.  Of long lattices the packing may need a cluster more than
+// counted here, and at such a line a whole round more, hence 2 % more.  The caller asks for 4 %
+// less than the launches' estimate: of 680 random batches of 4 to 1400 lattices 102 take clusters,
+// at 0.94 to 1.57 (eight below 1, mean 1.15) of the stretches' rate; front tests of 122 lattices
+// D1Q7 2.83 -> 2.24 us per step, D1Q5 2.06 -> 1.71.
 inline ClusterTiling choose_clusters(const std::vector<int64_t>& Ns, bool reservoir, int Q, int sms, int kwhole) {
-  const double t0 = Q == 7 ? 0.74 : 0.62, t1 = Q == 7 ? 0.085 : 0.064;
+  const double t0 = Q == 7 ? 0.68 : 0.63, t1 = Q == 7 ? 0.0975 : 0.071;
   const int C = (Q - 1) / 2;
   const std::vector<int64_t> n = length_sample(Ns, reservoir ? 2 * C : 0);
   const int64_t longest = n.front();
@@ -532,12 +534,18 @@ inline ClusterTiling choose_clusters(const std::vector<int64_t>& Ns, bool reserv
         if (b == room.size()) room.push_back(cap);
         room[b] -= std::max(v, pmin) + (v > NT ? pmin : pmin / 2);
       }
-      const double blocks = (double)room.size() * (double)Ns.size() / (double)n.size() * CL, per = (double)(768 / NT);
-      const double even = 0.95 * sms, hold = per * (cap > 1536 ? 0.85 : 0.95) * sms, full = std::floor(blocks / hold);
-      const double rest = std::ceil((blocks - full * hold) / even - 1e-9);
-      const double slow = cap > 1536 ? 1.15 : NT > 256 ? 1.08 : 1.0;
-      const auto step = [&](double b) { return slow * (t0 + t1 * std::max(b * NT / 32.0, 4.0)); };
-      const double us = full * step(per) + (rest > 0.0 ? step(rest) : 0.0) + 4.0 / kwhole;  // (a launch)
+      const double clusters = 1.02 * (double)room.size() * (double)Ns.size() / (double)n.size();
+      const auto hold = [&](int blocks) {  // clusters at once, with that many blocks an SM
+        const int small = sms / 16 * 2, large = (sms - 8 * small) / 2;  // (eight GPCs; those of two SMs more)
+        return (double)((8 - large) * (blocks * small / CL) + large * (blocks * (small + 2) / CL));
+      };
+      const int per = 768 / NT;
+      const double full = std::floor(clusters / std::max(1.0, hold(per))), rest = clusters - full * hold(per);
+      int blocks = 1;
+      while (blocks < per && hold(blocks) < rest - 1e-9) ++blocks;
+      const double slow = NT == 128 ? 1.0 : NT == 256 ? 1.09 : 1.1;
+      const auto step = [&](int b) { return slow * (t0 + t1 * std::max(b * NT / 32.0, 4.0)); };
+      const double us = full * step(per) + (rest > 1e-9 ? step(blocks) : 0.0) + 4.0 / kwhole;  // (a launch)
       if (us < best.us) best = ClusterTiling{NT, CL, us};
     }
   return best;
