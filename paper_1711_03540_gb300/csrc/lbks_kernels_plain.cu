@@ -151,9 +151,12 @@ __global__ void __launch_bounds__(kPlainThreads) gather_rho_kernel(Arena src, co
 }
 
 // The plain fused step: one thread per site reads its Q populations, collides
-// (Eq. LB_equation_ordinary) and pushes f*_i to site x + c_i (mod N).
+// (Eq. LB_equation_ordinary) and pushes f*_i to site x + c_i (mod N).  Bound by the latency of the
+// FP64 collision's integer chain, so by the warps of an SM: 32 with 64 registers a thread (D1Q7: 8
+// bytes of spills; it takes 96 of its own) step the 4096-lattice ensemble in 254 us (D1Q5 210), 24
+// in 310 (246), 16 in 379.
 template <int Q, int ST>
-__global__ void __launch_bounds__(kPlainThreads, ST == kF64 ? 3 : 1) plain_step_kernel(Arena src, Arena dst,
+__global__ void __launch_bounds__(kPlainThreads, ST == kF64 ? 4 : 1) plain_step_kernel(Arena src, Arena dst,
                                                                    const RunDesc* __restrict__ runs,
                                                                    const Tile* __restrict__ tiles) {
   using T = typename StorageType<ST>::type;
@@ -192,8 +195,11 @@ __global__ void __launch_bounds__(kPlainThreads, ST == kF64 ? 3 : 1) plain_step_
 // the f^eq(rho_bc) it holds) with the same collide() as every other kernel and
 // pushes plane i to j + c_i when that node is interior (pushes into reservoir
 // nodes are dropped), so each interior node receives exactly one value per plane.
+// (Registers as above; D1Q7 spills 40 bytes at 64 of them and small batches lose 3 %, so it keeps
+// 24 warps: 122 lattices 4.77 against 4.94 us, 1200 of 2000 sites 139 against 133; D1Q5 94 with 32
+// warps, 104 with 24.)
 template <int Q, int ST>
-__global__ void __launch_bounds__(kPlainThreads, ST == kF64 ? 3 : 1) reservoir_step_kernel(Arena src, Arena dst,
+__global__ void __launch_bounds__(kPlainThreads, ST != kF64 ? 1 : Q == 7 ? 3 : 4) reservoir_step_kernel(Arena src, Arena dst,
                                                                        const RunDesc* __restrict__ runs,
                                                                        const Tile* __restrict__ tiles, int reset_only) {
   using T = typename StorageType<ST>::type;
