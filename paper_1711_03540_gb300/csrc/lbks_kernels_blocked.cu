@@ -23,12 +23,11 @@
 // 1.12 us; 2^20 sites 3.1 against 2.2 us, so large FP32 batches stay register-resident.
 // Not for scaled FP16, whose results depend on where launches end (rounded there).
 // Per step and stretch: the halos cost 2 c_max k of NT sites, a launch 1.5 to 2 us in all.
-// Measured (GB300): one 4096-site D1Q7 FP64 lattice 16.8 -> 0.71 us per step (stretches of
+// Measured (GB300): one 4096-site D1Q7 FP64 lattice 16.8 -> 0.87 us per step (stretches of
 // 32 sites, 16 steps per launch; bound by the latency of one warp's collision), the
-// 4096-lattice FP64 ensemble 615 -> 209 us per step, 4.5e10 site-updates/s (128 threads, 2
-// steps per launch; bound by the integer pipe, 55 % busy, and the conversions, 56 %, which
-// contend; having L2 fetch the state a round of blocks ahead gave 0.6 %), 122 front lattices
-// 9.8 -> 2.2 us per step (over clusters; stretches 2.9), 24 FP32 lattices 0.87 -> 0.37 us per step.
+// 4096-lattice FP64 ensemble 615 -> 253 us per step, 3.7e10 site-updates/s (128 threads, 2
+// steps per launch; bound by the integer pipe, 65 % busy), 122 front lattices 9.8 -> 2.2 us per
+// step (over clusters), 24 FP32 lattices 0.87 -> 0.37 us per step.
 #include "lbks_collapse.cuh"
 #include "lbks_device.cuh"
 #include "lbks_plan.h"
@@ -71,16 +70,19 @@ template <int Q, int ST, int NTM> struct BlockedCfg {
 
 // ONE: every bundle holds one piece.  MINB: blocks an SM has to hold, which sets the
 // register budget: 80 in FP64 (24 warps), 64 in FP32 where SMs are to be filled; FP64 batches
-// of at most a block per SM take what the compiler wants instead (122), which shortens the
-// one warp per scheduler's chain by 4 to 6 %.
+// of at most a block per SM take what the compiler wants instead (about 126), which shortens the
+// one warp per scheduler's chain by 4 to 6 %.  Where a block holds several runs, their fixed-point
+// constants lie in shared memory and are read every step: in registers (uniform ones where the
+// block has one run) they were spilled, 152 bytes a thread (122 front lattices 2.70 -> 2.44 us
+// per step).
 // CLU: the blocks of a cluster hold lattices together (plan_clusters), without halos: a portion's
 // edge values are also stored into the guard columns of the block that holds its neighbour
 // (st.shared::cluster; the portion itself where a lattice lies in one block), and the step's barrier is
 // the cluster's.  For FP64 batches with lattices longer than a block: their stretches cost up
 // to two thirds more sites in halos, and launches that end block by block every 4 to 16
-// steps.  The cluster barrier adds 0.3 us to a step's latency (1.02 against 0.72 us with one
-// block an SM), which other blocks of the SM cover; 122 front lattices 2.86 -> 2.23 us per
-// step, 140 lattices of up to 1200 sites 3.55 -> 2.27 us, single lattices stay in stretches.
+// steps.  The cluster barrier adds 0.25 us to a step's latency (1.13 against 0.87 us with one
+// block an SM), which other blocks of the SM cover; 122 front lattices 2.83 -> 2.24 us per
+// step, single lattices stay in stretches.
 template <int Q, int ST, int NTM, int MINB, bool RES, bool ONE, bool CLU = false>
 __global__ void __launch_bounds__(NTM, MINB)
     blocked_step_kernel(Arena src, Arena dst, const RunDesc* __restrict__ runs, const Piece* __restrict__ pieces,
